@@ -163,27 +163,19 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     return fn;
 }
 
-// Tensor maps for TMA tile loads of phi and tile stores of labels: box (32, ty, tz),
-// zero fill outside the lattice.  TMA needs 16-byte aligned base addresses and row
-// pitches, so nx must be a multiple of 4; otherwise tm.valid stays 0 and the
-// kernels use cp.async loads and plain stores.
-void make_tmaps(const hk_lattice &l, int ty, int tz, hk::TmapPair &tm) {
+// Tensor map for TMA tile loads of phi: box (32, ty, tz), zero fill outside the lattice.
+// TMA needs a 16-byte aligned base address and row pitch, so nx must be a multiple of
+// 4; otherwise tm.valid stays 0 and the occupancy pass uses plain loads.
+void make_tmap(const hk_lattice &l, int ty, int tz, hk::PhiTmap &tm) {
     std::memset(&tm, 0, sizeof(tm));
     auto fn = encode_fn();
-    if (!fn || (l.nx % 4) != 0 || (reinterpret_cast<uintptr_t>(l.phi) & 15) ||
-        (reinterpret_cast<uintptr_t>(l.labels) & 15))
-        return;
+    if (!fn || (l.nx % 4) != 0 || (reinterpret_cast<uintptr_t>(l.phi) & 15)) return;
     const cuuint64_t dims[3] = {(cuuint64_t)l.nx, (cuuint64_t)l.ny, (cuuint64_t)l.nz};
     const cuuint64_t strides[2] = {(cuuint64_t)l.nx * 4, (cuuint64_t)l.nx * l.ny * 4};
     const cuuint32_t box[3] = {(cuuint32_t)hk::TX, (cuuint32_t)ty, (cuuint32_t)tz};
     const cuuint32_t estr[3] = {1, 1, 1};
     if (fn(&tm.phi, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float *>(l.phi), dims, strides, box, estr,
            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return;
-    // labels leave a staged tile laid out with the 128-byte swizzle (box rows are 128 bytes)
-    if (fn(&tm.labels, CU_TENSOR_MAP_DATA_TYPE_INT32, 3, l.labels, dims, strides, box, estr,
-           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return;
     tm.valid = 1;
@@ -420,8 +412,8 @@ int run_lattices(hk_ctx *ctx, const hk_lattice *lats, int n, cudaStream_t st, bo
             ev = ctx->ev[slot];
             ctx->ncalls += 1;
         }
-        std::vector<hk::TmapPair> tms(cn);
-        for (int i = 0; i < cn; ++i) make_tmaps(lats[c0 + i], ctx->ty, ctx->tz, tms[i]);
+        std::vector<hk::PhiTmap> tms(cn);
+        for (int i = 0; i < cn; ++i) make_tmap(lats[c0 + i], ctx->ty, ctx->tz, tms[i]);
         e = hk::launch_label(ctx->ty, ctx->tz, dev.data(), cn, P, W, tms.data(), st, ev, ctx->merge);
         if (e != cudaSuccess) return fail_cuda(ctx, e);
         if (inside && dev[0].sizes_cap > 0) {

@@ -1,5 +1,4 @@
-// hk_device.cuh -- device-side data structures, PTX helpers (TMA, mbarrier,
-// cp.async) and the union-find primitives of the labelling passes.
+// hk_device.cuh -- device-side data structures, PTX helpers (TMA, mbarrier) and the union-find primitives of the labelling passes.
 //
 // Tiles are 32 sites along x (one 32-bit occupancy word per tile row) by TY
 // rows along y by TZ planes along z.  Inside a tile the Hoshen-Kopelman raster
@@ -65,7 +64,8 @@ struct Work {
     uint32_t *pre;      // [nrows + 1] exclusive prefix of the roots per lattice row
     uint32_t *bsum;     // [nblocks] scan block sums
     uint16_t *face;     // [ntiles * face_stride] per-face lists of boundary-piece numbers
-    int4 *tinfo;        // [ntiles] (piece base, piece count, run count, 0) of each tile
+    int4 *tinfo;        // [ntiles] each tile's first site (x, y, z) and its counts: boundary pieces
+                        // (bits 0-10), runs (bits 11-23), lattice of the launch (bits 24-29)
     int32_t *parent;    // [piece_cap] union-find parent over boundary pieces; tile t owns
                         // the slice [t * MAX_BOUNDARY, t * MAX_BOUNDARY + piece count)
     int32_t *key;       // [piece_cap] lattice-local site index of the piece's first site;
@@ -91,11 +91,10 @@ struct Work {
     int32_t *roots;
 };
 
-// Tensor maps of the single-lattice fast path (TMA tile loads of phi and TMA
-// tile stores of labels).  Unused when `valid` is 0.
-struct TmapPair {
+// Tensor map of a lattice's phi (TMA tile loads of the occupancy pass).  Unused when
+// `valid` is 0.
+struct PhiTmap {
     CUtensorMap phi;
-    CUtensorMap labels;
     int valid;
 };
 
@@ -103,7 +102,7 @@ struct TmapPair {
 // by value).
 template <int NL>
 struct TmapBatch {
-    TmapPair tm[NL];
+    PhiTmap tm[NL];
 };
 
 // A union-find path longer than the number of its nodes means corrupted
@@ -204,6 +203,13 @@ __device__ __forceinline__ bool occupied(float v, int mode) { return mode ? (v <
 __device__ __forceinline__ uint32_t run_starts(uint32_t m) { return m & ~(m << 1); }
 // the last site of every run: bit x set when x is occupied and x + 1 is not (or x = 31)
 __device__ __forceinline__ uint32_t run_ends(uint32_t m) { return m & ~(m >> 1); }
+// position of the highest set bit of w (of the only one, for an isolated bit: one
+// instruction, where __ffs takes two on the same slow pipe)
+__device__ __forceinline__ int top_bit(uint32_t w) {
+    int p;
+    asm("bfind.u32 %0, %1;" : "=r"(p) : "r"(w));
+    return p;
+}
 // bits 0..x set
 __device__ __forceinline__ uint32_t le_mask(int x) { return (2u << x) - 1u; }
 // run id (within the tile) of occupied site x of a row with run starts rs
@@ -257,23 +263,6 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t b
                  ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar))
                  : "memory");
 }
-// TMA tile store; elements outside the tensor are not written.  Coordinates are never negative.
-__device__ __forceinline__ void tma_store_3d(const CUtensorMap *map, const void *src, int x, int y, int z) {
-    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
-                 ::"l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(src))
-                 : "memory");
-}
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_read0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait0() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-// 4-byte asynchronous global->shared copy; src_bytes == 0 writes a zero.
-__device__ __forceinline__ void cp_async4(void *dst, const void *src, int src_bytes) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(src_bytes)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
 // Wait for phase `parity` of an mbarrier with an iteration cap; returns false on timeout.
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity) {
     for (uint32_t it = 0; it < (1u << 26); ++it)

@@ -14,9 +14,8 @@
 //                     roots and count cluster roots per row segment.
 //   S1-S3 scan        exclusive prefix of the root counts: the compactified
 //                     cluster numbering 1..n of Sec. 2 in row-major order.
-//   K4 flatten        persistent: decode the run codes, write the labels
-//                     (staged in shared memory, TMA tensor stores), the sizes
-//                     in label order and the histogram.
+//   K4 flatten        persistent: decode the run codes, write the labels, the
+//                     sizes in label order and the histogram.
 #include <cstring>
 #include <mutex>
 #include <type_traits>
@@ -233,7 +232,8 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
 
     for (int64_t it = blockIdx.x; it < nwork; it += gridDim.x) {
         const int64_t t = FAST ? it : (int64_t)W.ovf[it];
-        const LatDev &L = B.lat[(NL == 1) ? 0 : find_lattice(B.lat, B.n, t)];
+        const int lat = (NL == 1) ? 0 : find_lattice(B.lat, B.n, t);
+        const LatDev &L = B.lat[lat];
         const TileGeo g = tile_geo<TY, TZ>(L, t);
 
         const int r = tid, ly = r % TY, lz = r / TY;
@@ -469,7 +469,9 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
             W.psize[pid] = S.aux[i] & (AUX_FACE - 1);
             S.aux[i] = -1 - k;                   // from here on: boundary root k
         }
-        if (tid == 0) W.tinfo[t] = make_int4(base, nb_, total, 0);
+        if (tid == 0)
+            W.tinfo[t] = make_int4(g.x0, g.y0, g.z0,
+                                   nb_ | (total << 11) | (lat << 24));
         __syncthreads();
 
         // interior roots per row segment (a row's runs span at most two chunks)
@@ -666,7 +668,7 @@ k_face_merge(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
 // --------------------------------------------------------------------------------------
 template <int NL, bool HOT>
 __global__ void __launch_bounds__(32 * PF_WARPS)
-k_piece_finalize(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
+k_piece_finalize(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles, int max_boundary) {
     grid_dep_wait();
     __shared__ int hot_target[PF_WARPS];   // per warp: the cluster root its pieces fed most, and the sum
     __shared__ int hot_sum[PF_WARPS];
@@ -675,13 +677,13 @@ k_piece_finalize(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles)
     // The root that collects most sizes (the percolating cluster's, above all) is added
     // once per warp and then once per CTA; other roots once per group of lanes.
     int hot = -1, hot_acc = 0;
-    const int4 ti = t < ntiles ? W.tinfo[t] : make_int4(0, 0, 0, 0);
-    if (ti.y > 0) {
+    const int nbnd = t < ntiles ? W.tinfo[t].w & 0x7ff : 0;
+    if (nbnd > 0) {
         const LatDev &L = B.lat[(NL == 1) ? 0 : find_lattice(B.lat, B.n, t)];
-        for (int j0 = 0; j0 < ti.y; j0 += 32) {
+        for (int j0 = 0; j0 < nbnd; j0 += 32) {
             const int j = j0 + lane;
-            const bool valid = j < ti.y;
-            const int pid = ti.x + j;
+            const bool valid = j < nbnd;
+            const int pid = (int)t * max_boundary + j;
             int root = -1, add = 0;
             if (valid) {
                 root = g_find_ro(W.parent, pid, W.piece_cap, W.status);
@@ -866,212 +868,331 @@ __global__ void k_lattice_finish(const __grid_constant__ LatBatch<NL> B, Work W)
 
 // --------------------------------------------------------------------------------------
 // K4: flatten (decode run codes; no union-find)
+//
+// Per tile: one thread per row numbers the row's runs (a block scan) and gives each run
+// its own first site as label; one thread per run then replaces that label unless the
+// run is the first of an interior piece (balanced over the threads whatever the rows
+// hold) and notes the cluster roots in a bitmap; one thread per row ranks its row's
+// roots and collects their sizes; and the labels leave, four sites a lane, straight to
+// global memory.  The next tile's record, words, codes and boundary pieces come by bulk
+// copy while the labels are written.
+//
+// Bound by instruction issue at p_c (1.2 warp instructions a site, 70 % of the issue
+// rate) and by the label stores on fields of long runs.  Against a loop over each row's
+// runs that decoded, ranked and filled them into a staged tile for a TMA store: 1.33
+// against 1.57 ms at 1024^3, p_c, 0.88 against 0.92 ms on blocks of 16^3, 0.105 against
+// 0.126 ms on a 512^3 bijel, 52 against 65 us at 387 x 283 x 221 (unaligned rows).
 // --------------------------------------------------------------------------------------
-// The staged tile uses the TMA 128-byte swizzle: in each tile row (128 bytes) the
-// 16-byte chunk index is XORed with the row index mod 8, so that threads writing the
-// same x of consecutive rows hit different banks.
-__device__ __forceinline__ int stage_idx(int row, int x) { return row * 32 + (x ^ ((row & 7) << 2)); }
-
+// Resident threads of an SM (40 registers each).  2048 (32 registers, spills): 1.63 ms at
+// 1024^3, p_c, against 1.50 for 1536 and 1.59 for 1280, in the form of that time.
+constexpr int FLAT_THREADS = 1536;
+// Items a CTA takes, each a stretch of consecutive tiles, so that a row's ranks and half
+// full size sectors carry over along x: 4 or 1 longer ones, 1.39 and 1.38 against 1.41 ms
+// at 1024^3, p_c, but 0.92 against 0.89 ms on blocks of 16^3, and a field whose parts
+// differ needs several to even out.
+constexpr int FLAT_ITEMS = 8;
 template <int TY, int TZ>
 struct FlatSmem {
     using SH = TileShape<TY, TZ>;
-    alignas(1024) int32_t stage[SH::SITES];   // labels [lz][ly][x], swizzled (TMA store source)
-    static constexpr int GL = SH::MAX_BOUNDARY < 384 ? SH::MAX_BOUNDARY : 384;   // staged boundary pieces
-    static_assert(GL % 4 == 0 && (SH::MAX_BOUNDARY * 4) % 16 == 0 && (SH::MAXRUNS * 2) % 16 == 0,
+    static constexpr int GL = SH::MAX_BOUNDARY < 256 ? SH::MAX_BOUNDARY : 256;   // staged boundary pieces
+    static constexpr int CC = SH::MR_FAST;                                       // staged run codes
+    static_assert(GL % 4 == 0 && CC % 8 == 0 && (SH::MAX_BOUNDARY * 4) % 16 == 0 && (SH::MAXRUNS * 2) % 16 == 0,
                   "bulk copies of whole 16-byte blocks from 16-byte aligned slices");
-    alignas(16) uint16_t codes[SH::MAXRUNS];  // the tile's run codes (bulk copy)
-    alignas(16) int gl[GL];                   // label of each boundary piece's cluster
-    alignas(16) int gsize[GL];                // cluster size if the piece is the cluster root, else -1
-    uint64_t bar;                             // completion of the tile's bulk copies
-    int warp_tmp[32];
+    // the staged tile (bulk copies)
+    alignas(16) uint32_t words[SH::R];         // occupancy word of each row
+    alignas(16) uint16_t codes[CC];            // run codes
+    // tab[0, GL): label of each boundary piece's cluster (copied); tab[GL, GL + R): first site of
+    // each row (computed)
+    // (an interior root's code holds a size, whose row is read but not used: one entry more)
+    alignas(16) int tab[GL + SH::R + 4];
+    alignas(16) int gsize[GL + 4];             // cluster size if the piece is the cluster root, else -1;
+                                               // [GL] = 1 stands for every interior piece
+    alignas(16) int4 tinfo;
+    uint64_t bar;                              // completion of the copies
+    uint4 row[SH::R];                          // occupancy word, run starts, first run id of each row
+    int lab[SH::MAXRUNS];                      // label of each run
+    uint32_t rootbal[SH::MAXRUNS / 32 + 1];    // cluster-root bits of each 32 run ids
+    alignas(16) int pend[SH::R][8];            // each row's sizes not yet written, by place in their sector
+                                               // (mod 8: two sectors)
+    int warp_tmp[SH::NT / 32];
     int hist[32];
 };
-
-template <int TY, int TZ>
-__device__ __forceinline__ int site_of(const TileGeo &g, const LatDev &L, int pos) {
-    const int row = pos >> 5, x = pos & 31;
-    return ((g.z0 + row / TY) * L.ny + (g.y0 + row % TY)) * L.nx + g.x0 + x;
-}
 
 // SLAB: one slab of a lattice split along z (W.site_off added to every label, each
 // cluster's label written to W.roots); a separate instance, so that the common path
 // carries neither.
 template <int TY, int TZ, int NL, bool SLAB>
-__global__ void __launch_bounds__(TY * TZ, 1280 / (TY * TZ))
-k_flatten(const __grid_constant__ LatBatch<NL> B, const __grid_constant__ TmapBatch<NL> TB, Work W, int64_t ntiles) {
+__global__ void __launch_bounds__(TY * TZ, FLAT_THREADS / (TY * TZ))
+k_flatten(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles, uint32_t span) {
     grid_dep_wait();
     using SH = TileShape<TY, TZ>;
-    constexpr int R = SH::R, NT = SH::NT, NW = NT / 32, MR = SH::MAXRUNS;
+    using FS = FlatSmem<TY, TZ>;
+    constexpr int R = SH::R, NT = SH::NT, NW = NT / 32, MR = SH::MAXRUNS, MB = SH::MAX_BOUNDARY;
+    constexpr int GL = FS::GL, CC = FS::CC;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    FlatSmem<TY, TZ> &S = *reinterpret_cast<FlatSmem<TY, TZ> *>(smem_raw);
+    FS &S = *reinterpret_cast<FS *>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    // the swizzled TMA store needs a 1024-byte aligned source; otherwise plain stores
-    const bool stage_ok = (smem_u32(S.stage) & 1023u) == 0;
 
     if (tid < 32) S.hist[tid] = 0;
+    if (tid == 0) S.gsize[GL] = 1;
+    // Thread 0 issues the copies of a tile (its record ti says how much there is).  If they
+    // do not complete within their bound the CTA records STATUS_TMA_TIMEOUT and stages
+    // its tiles by plain loads from then on (prefetch becomes false, uniformly).
+    auto issue = [&](uint32_t t, int4 ti) {
+        const int nb = ti.w & 0x7ff, total = (ti.w >> 11) & 0x1fff;
+        const int nc = min((total + 7) & ~7, CC), ng = min((nb + 3) & ~3, GL);
+        fence_proxy_async();
+        mbar_arrive_expect_tx(&S.bar, (uint32_t)(4 * R + 16 + 2 * nc + 8 * ng));
+        bulk_load(&S.tinfo, W.tinfo + t, 16u, &S.bar);
+        bulk_load(S.words, W.mask + (size_t)t * R, 4u * R, &S.bar);
+        if (nc) bulk_load(S.codes, W.codes + (size_t)t * MR, 2u * nc, &S.bar);
+        if (ng) {
+            bulk_load(S.tab, W.key + (size_t)t * MB, 4u * ng, &S.bar);
+            bulk_load(S.gsize, W.psize + (size_t)t * MB, 4u * ng, &S.bar);
+        }
+    };
+    // CTA b takes the tiles [i span, (i + 1) span) of every item i = b, b + gridDim.x, ...
+    const uint32_t nt = (uint32_t)ntiles, skip = (gridDim.x - 1u) * span;
+    auto next_tile = [&](uint32_t &t, uint32_t &end) {
+        if (++t >= end) {
+            t = end + skip;
+            end = t < nt ? min(t + span, nt) : t;
+        }
+    };
+    uint32_t t = blockIdx.x * span, end = min(t + span, nt);
+    bool fresh = true;                                 // uniform: the first tile of an item
+    int4 ti_next = make_int4(0, 0, 0, 0);              // thread 0: the record of the next tile
     if (tid == 0) {
         mbar_init(&S.bar, 1);
         fence_mbar_init();
+        // the first tile's counts are not waited for: all that can be staged is copied
+        if (t < nt) issue(t, make_int4(0, 0, 0, GL | (CC << 11)));
+        uint32_t t1 = t, e1 = end;
+        next_tile(t1, e1);
+        if (t1 < nt) ti_next = W.tinfo[t1];
     }
-    // The tile's run codes and its staged boundary-piece records arrive by bulk copies
-    // issued at the start of the tile, so that the run loop reads shared memory.  If a
-    // copy does not complete within its bound the CTA records STATUS_TMA_TIMEOUT and
-    // reads global memory from then on (prefetch becomes false, uniformly).
+    __syncthreads();
     bool prefetch = true;
-    int ktile = 0;
+    uint32_t parity = 0;
     int cur_lat = -1;
-    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x, ++ktile) {
-        const int lat = (NL == 1) ? 0 : find_lattice(B.lat, B.n, t);
-        const LatDev &L = B.lat[lat];
-        const TileGeo g = tile_geo<TY, TZ>(L, t);
-        const bool use_tma = TB.tm[lat].valid && stage_ok;
-        const int4 ti = W.tinfo[t];
-        const int base = ti.x, nb = ti.y;
-        const int r = tid, ly = r % TY, lz = r / TY;
-        const uint32_t m = W.mask[t * R + r];
-        const uint32_t rs = run_starts(m);
-        const bool valid_row = ly <= g.lastY && lz <= g.lastZ;
-        // rank base of this row: issued early, used after the barriers below
-        uint32_t pre_row = 0, pre_lat = 0;
-        if (rs && valid_row) {
-            // roots of the lattice's earlier rows, then of this row's earlier segments
-            const int64_t q = (int64_t)(g.z0 + lz) * L.ny + (g.y0 + ly);
-            pre_row = W.pre[L.row0 + q] + bytes_sum(W.cnt, L.seg0 + q * L.nbx, g.bx);
-            pre_lat = W.pre[L.row0];
-        }
-
-        const uint16_t *C = W.codes + t * MR;
-        constexpr int GL = FlatSmem<TY, TZ>::GL;
-        if (tid == 0) bulk_wait_read0();               // a previous tile's store has read S.stage
-        __syncthreads();                               // ... and every thread is done with S.codes, S.gl
-        if (prefetch && tid == 0) {
-            const int ncode = (ti.z + 7) & ~7;                       // whole 16-byte blocks
-            const int ng = ((nb < GL ? nb : GL) + 3) & ~3;
-            mbar_arrive_expect_tx(&S.bar, (uint32_t)(2 * ncode + 8 * ng));
-            if (ncode) bulk_load(S.codes, C, 2u * ncode, &S.bar);
-            if (ng) {
-                bulk_load(S.gl, W.key + base, 4u * ng, &S.bar);
-                bulk_load(S.gsize, W.psize + base, 4u * ng, &S.bar);
+    uint32_t rank = 0, lo = 0;                         // of this row: next rank, first one not written
+    while (t < nt) {
+        uint32_t m, rs;
+        int inc;
+        for (;;) {
+            bool done = true;
+            if (prefetch) {
+                done = mbar_wait_bounded(&S.bar, parity);
+            } else {
+                const int4 ti = W.tinfo[t];
+                const int nb = ti.w & 0x7ff, total = (ti.w >> 11) & 0x1fff;
+                if (tid == 0) S.tinfo = ti;
+                S.words[tid] = W.mask[(size_t)t * R + tid];
+                for (int k = tid; k < total && k < CC; k += NT) S.codes[k] = W.codes[(size_t)t * MR + k];
+                for (int k = tid; k < nb && k < GL; k += NT) {
+                    S.tab[k] = W.key[(size_t)t * MB + k];
+                    S.gsize[k] = W.psize[(size_t)t * MB + k];
+                }
             }
+            m = S.words[tid];
+            rs = run_starts(m);
+            inc = __popc(rs);                          // run ids: inclusive scan over the warp's rows
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, inc, d);
+                if (lane >= d) inc += u;
+            }
+            if (lane == 31) S.warp_tmp[wid] = inc;
+            if (!__syncthreads_or(!done)) break;       // ... and every thread is done with S.row, S.lab
+            if (tid == 0) atomicOr(W.status, STATUS_TMA_TIMEOUT);
+            mbar_wait_bounded(&S.bar, parity);         // the copies still in flight
+            prefetch = false;
+        }
+        parity ^= 1;
+        const int4 ti = S.tinfo;
+        const int nb = ti.w & 0x7ff, total = (ti.w >> 11) & 0x1fff, lat = NL == 1 ? 0 : ti.w >> 24;
+        const LatDev &L = B.lat[lat];
+        const int r = tid, ly = r % TY, lz = r / TY;
+        // Rank base of this row: the roots of the lattice's earlier rows, then of this row's
+        // earlier segments; carried on while the tiles follow each other along x.
+        const int q = (ti.z + lz) * L.ny + (ti.y + ly);
+        const bool valid_row = ti.y + ly < L.ny && ti.z + lz < L.nz;
+        if ((fresh || ti.x == 0) && valid_row) {
+            rank = W.pre[L.row0 + q] - W.pre[L.row0];
+            if (ti.x) rank += bytes_sum(W.cnt, L.seg0 + (int64_t)q * L.nbx, ti.x / TX);
+            lo = rank;
         }
         if (lat != cur_lat) {                          // uniform: flush the histogram per lattice
             if (cur_lat >= 0 && tid < 32 && S.hist[tid] && B.lat[cur_lat].hist)
                 atomicAdd(reinterpret_cast<unsigned long long *>(B.lat[cur_lat].hist) + tid,
                           (unsigned long long)S.hist[tid]);
-            __syncthreads();
             if (tid < 32) S.hist[tid] = 0;
             cur_lat = lat;
         }
+        int rb = inc - __popc(rs);
+#pragma unroll
+        for (int w = 0; w < NW; ++w)
+            if (w < wid) rb += S.warp_tmp[w];
+        S.row[r] = make_uint4(m, rs, (uint32_t)rb, 0u);
 
-        for (int i = tid; i < SH::SITES / 4; i += NT)
-            reinterpret_cast<int4 *>(S.stage)[i] = make_int4(-1, -1, -1, -1);
-        int tot2;
-        const int rb = block_exscan<NT>(__popc(rs), S.warp_tmp, tot2);   // ends with a barrier
-        if (prefetch) {
-            const bool done = mbar_wait_bounded(&S.bar, (uint32_t)(ktile & 1));
-            if (__syncthreads_or(!done)) {             // uniform: give up the prefetch
-                if (tid == 0) atomicOr(W.status, STATUS_TMA_TIMEOUT);
-                mbar_wait_bounded(&S.bar, (uint32_t)(ktile & 1));   // the copies still in flight
-                prefetch = false;
-            }
-        }
-        if (!prefetch) {                               // staged by the threads instead
-            for (int k = tid; k < nb && k < GL; k += NT) {
-                S.gl[k] = __ldg(W.key + base + k);       // cluster label (written by piece_finalize)
-                S.gsize[k] = __ldg(W.psize + base + k);  // cluster size at the root piece, else -1
-            }
-            __syncthreads();
-        }
-
-        // a4-a7: one pass over the runs of each row in x order: cluster roots get
-        // their rank, size and histogram entry; every run writes its label.  The loop
-        // is compiled for each case of two tile-uniform conditions, so that neither is
-        // tested per run: PF, the codes and piece records arrived by bulk copy (else
-        // they are read from global memory); BIG, the tile has boundary pieces beyond
-        // the staged ones (read from global memory).
-        int64_t rank = (int64_t)(uint32_t)(pre_row - pre_lat);
-        const int site_row = ((g.z0 + lz) * L.ny + (g.y0 + ly)) * L.nx + g.x0;
-        const int site_row0 = (g.z0 * L.ny + g.y0) * L.nx + g.x0, sxy_i = L.nx * L.ny;
-        uint32_t rootbits = 0;                // first sites of cluster roots in this row
+        // every run starts with its own first site as label
         const int soff = SLAB ? (int)W.site_off : 0;   // labels of a slab are sites of the whole lattice
-        const uint32_t re = run_ends(m);
-        auto run_loop = [&](auto PF, auto BIG) {
-            constexpr bool pf = decltype(PF)::value, big = decltype(BIG)::value;
-            uint32_t w = rs;
-            int id = rb;
-            while (w) {
-                const int x0 = __ffs(w) - 1;
-                w &= w - 1;
-                const int c = pf ? (int)S.codes[id] : (int)__ldg(C + id);
-                ++id;
+        const int site_row = q * L.nx + ti.x + soff;
+        S.tab[GL + r] = site_row;
+        {
+            int *lp = S.lab + rb;
+            for (uint32_t w = rs; w;) {
+                const uint32_t low = w & (0u - w);
+                w ^= low;
+                *lp++ = site_row + top_bit(low);
+            }
+        }
+        __syncthreads();
+
+        // The next two steps are compiled for tiles that are staged whole and for others.
+        const uint16_t *C = W.codes + (size_t)t * MR;
+        const int32_t *gl_g = W.key + (size_t)t * MB, *gs_g = W.psize + (size_t)t * MB;
+        auto decode_runs = [&](auto BIG) {
+            constexpr bool big = decltype(BIG)::value;
+            // one run per thread: the label of its boundary piece's cluster, or of the first
+            // run of its interior piece; and whether it is its cluster's first run.  The
+            // pieces' labels and the rows' first sites are one table (tab), and gsize ends
+            // with a positive entry for the interior pieces, so that nothing branches; the
+            // lanes past the last run repeat it.
+            for (int i0 = wid * 32; i0 < total; i0 += NT) {
+                const int i = i0 + lane, ic = min(i, total - 1);
+                const int c = (!big || ic < CC) ? (int)S.codes[ic] : (int)__ldg(C + ic);
                 const int k = c & CODE_LOW;
-                const bool isb = (c & CODE_BOUNDARY) != 0, isr = (c & CODE_ROOT) != 0;
-                const int kk = k < FlatSmem<TY, TZ>::GL ? k : 0;
-                int gl = S.gl[kk], gs = S.gsize[kk];
-                if (big && isb && k >= FlatSmem<TY, TZ>::GL) {
-                    gl = __ldg(W.key + base + k);
-                    gs = __ldg(W.psize + base + k);
+                const bool isb = (c & CODE_BOUNDARY) != 0;
+                int lab, gs;
+                if (big && isb && k >= GL) {
+                    lab = __ldg(gl_g + k);
+                    gs = __ldg(gs_g + k);
+                } else {
+                    lab = S.tab[isb ? k : GL + (k >> 5)];
+                    gs = S.gsize[isb ? k : GL];
                 }
-                // all three labels are formed and one is selected (no divergent branches)
-                const int ci = (isb || isr) ? 0 : c;   // an interior non-root run: its root's position
-                const int crow = ci >> 5;
-                const int own = site_row + x0;
-                const int other = site_row0 + (crow / TY) * sxy_i + (crow % TY) * L.nx + (ci & 31);
-                const int lab = SLAB ? (isb ? gl : (isr ? own : other)) + soff : (isb ? gl : (isr ? own : other));
-                const int size = isr ? (isb ? gs : k) : -1;
-                if (size > 0) {
-                    if (rank < L.sizes_cap) {
-                        L.sizes[rank] = size;
-                        if (SLAB) W.roots[rank] = lab;
-                    }
-                    ++rank;
-                    rootbits |= 1u << x0;
-                    atomicAdd(&S.hist[31 - __clz(size)], 1);
-                }
-                const int xe = x0 + __ffs(re >> x0);   // one past the run's last site
-                int *row = S.stage + r * 32;
-                const int sw = (r & 7) << 2;
-                row[x0 ^ sw] = lab;
-#pragma unroll 1
-                for (int x = x0 + 1; x < xe; ++x) row[x ^ sw] = lab;
+                lab += isb ? soff : (k & 31);          // piece labels are sites of the slab
+                if ((c & (CODE_BOUNDARY | CODE_ROOT)) != CODE_ROOT) S.lab[i] = lab;
+                const uint32_t bal = __ballot_sync(0xffffffffu, gs > 0 && (c & CODE_ROOT));
+                if (lane == 0) S.rootbal[i0 >> 5] = bal;
             }
         };
-        if (!prefetch) run_loop(std::false_type{}, std::true_type{});
-        else if (nb > FlatSmem<TY, TZ>::GL) run_loop(std::true_type{}, std::true_type{});
-        else run_loop(std::true_type{}, std::false_type{});
-        if (L.inside && ly <= g.lastY && lz <= g.lastZ)   // index fields: ranks of any root, later
-            W.rootbits[L.seg0 + ((int64_t)(g.z0 + lz) * L.ny + (g.y0 + ly)) * L.nbx + g.bx] = rootbits;
-        if (use_tma) fence_proxy_async();
+        const bool big = total > CC || nb > GL;        // uniform
+        if (big) decode_runs(std::true_type{});
+        else decode_runs(std::false_type{});
         __syncthreads();
-        if (use_tma) {
-            if (tid == 0) {
-                tma_store_3d(&TB.tm[lat].labels, S.stage, g.x0, g.y0, g.z0);
-                bulk_commit();
-            }
-        } else if (g.lastX == TX - 1 && (L.nx & 3) == 0 && (reinterpret_cast<uintptr_t>(L.labels) & 15) == 0) {
-            // whole rows at 16-byte aligned addresses: lane l stores 4 labels (x = 4 (l % 8)
-            // .. + 3) of row l / 8 of each group of 4 rows (the swizzle keeps them together)
-            const int64_t sxy = (int64_t)L.nx * L.ny;
-            const int x4 = (lane & 7) * 4;
-            int32_t *out = L.labels + (int64_t)g.z0 * sxy + (int64_t)g.y0 * L.nx + g.x0 + x4;
-            for (int r4 = wid * 4; r4 < R; r4 += NW * 4) {
-                const int rr = r4 + (lane >> 3), yy = rr % TY, zz = rr / TY;
-                if (yy <= g.lastY && zz <= g.lastZ)
-                    __stcs(reinterpret_cast<int4 *>(out + (int64_t)zz * sxy + (int64_t)yy * L.nx),
-                           *reinterpret_cast<const int4 *>(S.stage + rr * 32 + (x4 ^ ((rr & 7) << 2))));
-            }
-        } else {
-            const int64_t sxy = (int64_t)L.nx * L.ny;
-            int32_t *out = L.labels + (int64_t)g.z0 * sxy + (int64_t)g.y0 * L.nx + g.x0 + lane;
-            if (lane <= g.lastX)
-                for (int rr = wid; rr < R; rr += NW) {
-                    const int yy = rr % TY, zz = rr / TY;
-                    if (yy <= g.lastY && zz <= g.lastZ)
-                        __stcs(out + (int64_t)zz * sxy + (int64_t)yy * L.nx, S.stage[stage_idx(rr, lane)]);
+
+        // a4, a6, a7: the roots of each row in x order get their ranks, sizes and
+        // histogram entries
+        const int n = __popc(rs);
+        uint32_t bits = 0;                             // the row's runs are bits 0 .. n - 1 (n <= 16)
+        if (n) bits = __funnelshift_r(S.rootbal[rb >> 5], S.rootbal[(rb >> 5) + 1], (uint32_t)rb & 31u) &
+                      ((1u << n) - 1u);
+        if (L.inside) {                                // index fields: ranks of any root, later
+            uint32_t rootbits = 0;                     // first sites of cluster roots in this row
+            for (uint32_t w = bits; w; w &= w - 1u) rootbits |= 1u << (S.lab[rb + __ffs(w) - 1] - site_row);
+            if (valid_row) W.rootbits[L.seg0 + (int64_t)q * L.nbx + ti.x / TX] = rootbits;
+        }
+        // Sizes wait in shared memory until their 32-byte sector is full (a row has fewer roots
+        // in a tile than that; the next tile along x brings the rest): stores of single
+        // sizes left part-written sectors that cost flatten 0.3 to 0.45 ms at 1024^3, p_c.
+        const uint32_t cap = (uint32_t)min(L.sizes_cap, (int64_t)INT32_MAX);   // ranks stay below 2^30
+        const uint32_t place = (uint32_t)(reinterpret_cast<uintptr_t>(L.sizes) >> 3);
+        auto flush = [&](bool all) {                   // the full sectors among ranks lo .. rank - 1, or all
+            while (lo < rank) {
+                const uint32_t e = lo + 4u - ((lo + place) & 3u);   // the first rank of the next sector
+                if (e > rank && !all) break;
+                if (e - lo == 4u && e <= rank && e <= cap) {
+                    const int4 p = *reinterpret_cast<const int4 *>(&S.pend[r][(lo + place) & 7u]);
+                    longlong2 *to = reinterpret_cast<longlong2 *>(L.sizes + lo);
+                    to[0] = make_longlong2(p.x, p.y);
+                    to[1] = make_longlong2(p.z, p.w);
+                    lo = e;
+                } else {
+                    const uint32_t last = min(e, rank);
+                    for (; lo < last; ++lo)
+                        if (lo < cap) L.sizes[lo] = S.pend[r][(lo + place) & 7u];
                 }
+            }
+        };
+        auto write_roots = [&](auto BIG) {
+            constexpr bool bigt = decltype(BIG)::value;
+            while (bits) {
+                do {
+                    const uint32_t low = bits & (0u - bits);
+                    bits ^= low;
+                    const int id = rb + top_bit(low);
+                    const int c = (!bigt || id < CC) ? (int)S.codes[id] : (int)__ldg(C + id);
+                    const int k = c & CODE_LOW;
+                    const bool isb = (c & CODE_BOUNDARY) != 0;
+                    const int gs = (bigt && isb && k >= GL) ? __ldg(gs_g + k) : S.gsize[isb ? k : GL];
+                    const int size = isb ? gs : k;
+                    if (SLAB && rank < cap) W.roots[rank] = S.lab[id];   // a root's label is its own first site
+                    S.pend[r][(rank + place) & 7u] = size;
+                    atomicAdd(&S.hist[top_bit((uint32_t)size)], 1);
+                    ++rank;
+                } while (bits && rank - lo < 8u);
+                flush(false);
+            }
+        };
+        if (big) write_roots(std::true_type{});
+        else write_roots(std::false_type{});
+        const uint32_t t_done = t;
+        next_tile(t, end);
+        fresh = t != t_done + 1u;
+        if (fresh || ti.x + TX >= L.nx) flush(true);
+        __syncthreads();                               // every thread is done with the staged tile
+        if (tid == 0 && prefetch && t < nt) {
+            issue(t, ti_next);
+            uint32_t t1 = t, e1 = end;
+            next_tile(t1, e1);
+            if (t1 < nt) ti_next = W.tinfo[t1];
+        }
+
+        // a5: the labels.  Rows of whole 16-byte blocks: lane l writes sites x4 = 4 (l % 8) .. + 3
+        // of row l / 8 of each group of 4 rows.  The warps step through the rows by whole
+        // planes, so that y stays and z grows.  Other rows: one site a lane.
+        constexpr int ZS = NW * 4 / TY;
+        static_assert(ZS >= 1 && ZS * TY == NW * 4, "the warps' rows fill whole planes");
+        const int64_t sxy = (int64_t)L.nx * L.ny;
+        const int nrow = min(TZ, L.nz - ti.z) * TY;    // rows of the tile's planes inside the lattice
+        if ((L.nx & 3) == 0 && (reinterpret_cast<uintptr_t>(L.labels) & 15) == 0) {
+            const int x4 = (lane & 7) * 4;
+            const int row0 = wid * 4 + (lane >> 3), y = ti.y + row0 % TY;
+            const uint32_t below = (1u << x4) - 1u;
+            int32_t *out = L.labels + (int64_t)(ti.z + row0 / TY) * sxy + (int64_t)y * L.nx + ti.x + x4;
+            if (y < L.ny && ti.x + x4 < L.nx)
+#pragma unroll 2
+                for (int row = row0; row < nrow; row += NW * 4, out += ZS * sxy) {
+                    const uint4 w = S.row[row];
+                    const uint32_t mm = w.x >> x4, ss = w.y >> x4;
+                    const int *lp = S.lab + (int)w.z - 1 + __popc(w.y & below);   // the last run that starts below x4
+                    int4 v = make_int4(-1, -1, -1, -1);
+                    if (ss & 1u) ++lp;
+                    if (mm & 1u) v.x = *lp;
+                    if (ss & 2u) ++lp;
+                    if (mm & 2u) v.y = *lp;
+                    if (ss & 4u) ++lp;
+                    if (mm & 4u) v.z = *lp;
+                    if (ss & 8u) ++lp;
+                    if (mm & 8u) v.w = *lp;
+                    __stcs(reinterpret_cast<int4 *>(out), v);
+                }
+        } else if (ti.x + lane < L.nx) {
+            const uint32_t le = le_mask(lane), me = 1u << lane;
+            for (int yy = wid; yy < TY && ti.y + yy < L.ny; yy += NW) {
+                int32_t *out = L.labels + (int64_t)ti.z * sxy + (int64_t)(ti.y + yy) * L.nx + ti.x + lane;
+#pragma unroll 4
+                for (int row = yy; row < nrow; row += TY, out += sxy) {
+                    const uint4 w = S.row[row];
+                    int v = S.lab[(int)w.z - 1 + __popc(w.y & le)];
+                    if (!(w.x & me)) v = -1;
+                    __stcs(out, v);
+                }
+            }
         }
     }
-    if (tid == 0) bulk_wait0();
     __syncthreads();
     if (cur_lat >= 0 && tid < 32 && S.hist[tid] && B.lat[cur_lat].hist)
         atomicAdd(reinterpret_cast<unsigned long long *>(B.lat[cur_lat].hist) + tid, (unsigned long long)S.hist[tid]);
@@ -1373,14 +1494,14 @@ static int persistent_grid(K kernel, int threads, size_t smem, int64_t ntiles) {
 }
 
 template <int TY, int TZ, int NL>
-static cudaError_t launch_all(const LatDev *lats, int n, const Plan &P, const Work &W, const TmapPair *tms,
+static cudaError_t launch_all(const LatDev *lats, int n, const Plan &P, const Work &W, const PhiTmap *tms,
                               cudaStream_t st, cudaEvent_t *ev, MergeSchedule ms) {
     using SH = TileShape<TY, TZ>;
     LatBatch<NL> B;
     B.n = n;
     B.pad_ = 0;
     for (int i = 0; i < n; ++i) B.lat[i] = lats[i];
-    // tensor maps: the TMA occupancy pass needs every lattice's; flatten picks per tile
+    // tensor maps: the TMA occupancy pass needs every lattice's
     TmapBatch<NL> TB;
     std::memset(&TB, 0, sizeof(TB));
     bool all_tma = n > 0 && tms != nullptr;
@@ -1433,6 +1554,7 @@ static cudaError_t launch_all(const LatDev *lats, int n, const Plan &P, const Wo
         grid0 = c[2];
     }
     const unsigned g4 = (unsigned)(P.ntiles < grid4 ? P.ntiles : grid4);
+    const uint32_t span4 = (uint32_t)((P.ntiles + (int64_t)grid4 * FLAT_ITEMS - 1) / ((int64_t)grid4 * FLAT_ITEMS));
     auto mark = [&](int i) { if (ev) cudaEventRecord(ev[i], st); };
     launch_error = cudaSuccess;
     mark(0);
@@ -1453,9 +1575,10 @@ static cudaError_t launch_all(const LatDev *lats, int n, const Plan &P, const Wo
     else if (ms.unions == 4) launch_dep(k_face_merge<TY, TZ, NL, 4>, gfm, 32 * FM_WARPS, 0, st, B, W, P.ntiles);
     else launch_dep(k_face_merge<TY, TZ, NL, 2>, gfm, 32 * FM_WARPS, 0, st, B, W, P.ntiles);
     mark(3);
+    constexpr int MB = SH::MAX_BOUNDARY;
     const unsigned gpf = (unsigned)((P.ntiles + PF_WARPS - 1) / PF_WARPS);
-    if (ms.hot) launch_dep(k_piece_finalize<NL, true>, gpf, 32 * PF_WARPS, 0, st, B, W, P.ntiles);
-    else launch_dep(k_piece_finalize<NL, false>, gpf, 32 * PF_WARPS, 0, st, B, W, P.ntiles);
+    if (ms.hot) launch_dep(k_piece_finalize<NL, true>, gpf, 32 * PF_WARPS, 0, st, B, W, P.ntiles, MB);
+    else launch_dep(k_piece_finalize<NL, false>, gpf, 32 * PF_WARPS, 0, st, B, W, P.ntiles, MB);
     mark(4);
     const int64_t nb = (P.nrows + SCAN_CH) / SCAN_CH;   // covers index nrows (the total)
     launch_dep(k_scan_reduce<NL>, (unsigned)nb, SCAN_NT, 0, st, B, (const uint8_t *)W.cnt, P.nrows, W.bsum);
@@ -1466,10 +1589,10 @@ static cudaError_t launch_all(const LatDev *lats, int n, const Plan &P, const Wo
     launch_dep(k_lattice_finish<NL>, (unsigned)n, 32u, 0, st, B, W);
     mark(6);
     if constexpr (NL == 1) {
-        if (W.roots || W.site_off) launch_dep(k_flatten<TY, TZ, NL, true>, g4, SH::NT, smem4, st, B, TB, W, P.ntiles);
-        else launch_dep(k_flatten<TY, TZ, NL, false>, g4, SH::NT, smem4, st, B, TB, W, P.ntiles);
+        if (W.roots || W.site_off) launch_dep(k_flatten<TY, TZ, NL, true>, g4, SH::NT, smem4, st, B, W, P.ntiles, span4);
+        else launch_dep(k_flatten<TY, TZ, NL, false>, g4, SH::NT, smem4, st, B, W, P.ntiles, span4);
     } else {
-        launch_dep(k_flatten<TY, TZ, NL, false>, g4, SH::NT, smem4, st, B, TB, W, P.ntiles);
+        launch_dep(k_flatten<TY, TZ, NL, false>, g4, SH::NT, smem4, st, B, W, P.ntiles, span4);
     }
     mark(7);
     if (launch_error != cudaSuccess) return launch_error;
@@ -1477,7 +1600,7 @@ static cudaError_t launch_all(const LatDev *lats, int n, const Plan &P, const Wo
 }
 
 template <int TY, int TZ>
-static cudaError_t launch_shape(const LatDev *lats, int n, const Plan &P, const Work &W, const TmapPair *tms,
+static cudaError_t launch_shape(const LatDev *lats, int n, const Plan &P, const Work &W, const PhiTmap *tms,
                                 cudaStream_t st, cudaEvent_t *ev, MergeSchedule ms) {
     if (n == 1) return launch_all<TY, TZ, 1>(lats, n, P, W, tms, st, ev, ms);
     return launch_all<TY, TZ, MAX_LAT_PER_LAUNCH>(lats, n, P, W, tms, st, ev, ms);
@@ -1502,7 +1625,7 @@ bool tile_info(int ty, int tz, TileInfo &ti) {
     return false;
 }
 
-cudaError_t launch_label(int ty, int tz, const LatDev *lats, int n, const Plan &P, const Work &W, const TmapPair *tms,
+cudaError_t launch_label(int ty, int tz, const LatDev *lats, int n, const Plan &P, const Work &W, const PhiTmap *tms,
                          cudaStream_t st, cudaEvent_t *ev, MergeSchedule ms) {
     if (ty == 8 && tz == 8) return launch_shape<8, 8>(lats, n, P, W, tms, st, ev, ms);
     if (ty == 16 && tz == 8) return launch_shape<16, 8>(lats, n, P, W, tms, st, ev, ms);

@@ -9,7 +9,7 @@ namespace hk {
 
 struct LatDev;
 struct Work;
-struct TmapPair;
+struct PhiTmap;
 
 // lattices per launch: the descriptors and tensor maps of a launch travel as kernel
 // parameters (under the 32 KB parameter limit)
@@ -109,10 +109,9 @@ struct MergeSchedule {
 };
 
 // ev: NUM_PASSES + 1 events recorded around the passes, or nullptr.  tms: the tensor
-// maps of each of the n lattices (valid == 0: that lattice takes the plain-load and
-// plain-store paths), or nullptr for none.
+// maps of each of the n lattices (valid == 0: the call takes the plain-load occupancy pass), or nullptr for none.
 cudaError_t launch_label(int ty, int tz, const LatDev *lats, int n, const Plan &P, const Work &W,
-                         const TmapPair *tms, cudaStream_t st, cudaEvent_t *ev, MergeSchedule ms = MergeSchedule());
+                         const PhiTmap *tms, cudaStream_t st, cudaEvent_t *ev, MergeSchedule ms = MergeSchedule());
 
 // The slab merge (hk_slab.cu): the face data of all R ranks and this rank's slab.
 struct SlabMerge {

@@ -113,7 +113,7 @@ extern "C" int hk_label_noalloc(const float *phi, int nx, int ny, int nz, const 
     d.seg0 = 0;
     d.row0 = 0;
 
-    hk::TmapPair tm;
+    hk::PhiTmap tm;
     std::memset(&tm, 0, sizeof(tm));   // plain-load path: no tensor maps
     cudaError_t e = hk::launch_label(TY, TZ, &d, 1, P, W, &tm, st, nullptr);
     if (e != cudaSuccess) return HK_ERR_CUDA;
