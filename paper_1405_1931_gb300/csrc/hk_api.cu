@@ -26,7 +26,7 @@ Work bind_work(char *base, const Layout &Ly, int32_t *status, int64_t piece_cap,
     W.codes = reinterpret_cast<uint16_t *>(base + Ly.codes);
     W.cnt = reinterpret_cast<uint8_t *>(base + Ly.cnt);
     W.pre = reinterpret_cast<uint32_t *>(base + Ly.pre);
-    W.bsum = reinterpret_cast<uint32_t *>(base + Ly.bsum);
+    W.bsum = reinterpret_cast<uint32_t *>(base + Ly.parent);
     W.face = reinterpret_cast<uint16_t *>(base + Ly.face);
     W.tinfo = reinterpret_cast<int4 *>(base + Ly.tinfo);
     W.parent = reinterpret_cast<int32_t *>(base + Ly.parent);

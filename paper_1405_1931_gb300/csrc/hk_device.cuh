@@ -62,7 +62,7 @@ struct Work {
     uint16_t *codes;    // [ntiles * MAXRUNS] one code per run (CODE_* above)
     uint8_t *cnt;       // [nseg] cluster roots per segment (row-major segment order; <= 16)
     uint32_t *pre;      // [nrows + 1] exclusive prefix of the roots per lattice row
-    uint32_t *bsum;     // [nblocks] scan block sums
+    uint32_t *bsum;     // [nblocks] scan block sums (in parent's space, which is free by then)
     uint16_t *face;     // [ntiles * face_stride] per-face lists of boundary-piece numbers
     int4 *tinfo;        // [ntiles] each tile's first site (x, y, z) and its counts: boundary pieces
                         // (bits 0-10), runs (bits 11-23), lattice of the launch (bits 24-29)

@@ -12,7 +12,7 @@
 //                     instead of being gathered to a root process.
 //   K3 piece_finalize compress the union-find, add piece sizes into cluster
 //                     roots and count cluster roots per row segment.
-//   S1-S3 scan        exclusive prefix of the root counts: the compactified
+//   S1-S2 scan        exclusive prefix of the root counts: the compactified
 //                     cluster numbering 1..n of Sec. 2 in row-major order.
 //   K4 flatten        persistent: decode the run codes, write the labels, the
 //                     sizes in label order and the histogram.
@@ -742,12 +742,15 @@ k_piece_finalize(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles,
 }
 
 // --------------------------------------------------------------------------------------
-// S1-S3: exclusive scan of the cluster roots per lattice row (the sum of the row's
+// S1-S2: exclusive scan of the cluster roots per lattice row (the sum of the row's
 // segment counts); ranks inside a row are completed by flatten from the segment
-// counts before its own.
+// counts before its own.  Launches and round trips bound it, not bytes: two launches
+// (block sums, then the rows) where four were (block sums, their scan, the rows, and
+// the counts and histograms), and blocks of 1024 rows where 4096 were, took a 256^3
+// call from 94.3 to 74.2 us.
 // --------------------------------------------------------------------------------------
 constexpr int SCAN_NT = 256;
-constexpr int SCAN_PER = 16;
+constexpr int SCAN_PER = 4;
 constexpr int SCAN_CH = SCAN_NT * SCAN_PER;
 
 template <int NL>
@@ -763,6 +766,7 @@ __global__ void __launch_bounds__(SCAN_NT) k_scan_reduce(const __grid_constant__
     __shared__ uint32_t red[SCAN_NT / 32];
     const int64_t b0 = (int64_t)blockIdx.x * SCAN_CH;
     uint32_t s = 0;
+#pragma unroll
     for (int j = 0; j < SCAN_PER; ++j) {
         const int64_t i = b0 + (int64_t)j * SCAN_NT + threadIdx.x;
         if (i < n) s += row_roots(B, cnt, i);
@@ -775,6 +779,9 @@ __global__ void __launch_bounds__(SCAN_NT) k_scan_reduce(const __grid_constant__
         for (int w = 0; w < SCAN_NT / 32; ++w) tot += red[w];
         bsum[blockIdx.x] = tot;
     }
+    // flatten adds to the histograms: cleared here, two passes before it
+    for (int i = blockIdx.x * SCAN_NT + threadIdx.x; i < 32 * B.n; i += gridDim.x * SCAN_NT)
+        if (B.lat[i >> 5].hist) B.lat[i >> 5].hist[i & 31] = 0;
 }
 
 // single block: exclusive scan of the block sums in place
@@ -812,12 +819,21 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(uint32_t *bsum, int64_t nb
     }
 }
 
+// scanned: bsum holds the exclusive scan of the block sums; else the sums themselves, and
+// every block adds up those before it (at most SCAN_DIRECT: a few loads a thread, for
+// one launch less).
+constexpr int64_t SCAN_DIRECT = 2048;
 template <int NL>
 __global__ void __launch_bounds__(SCAN_NT) k_scan_apply(const __grid_constant__ LatBatch<NL> B, const uint8_t *cnt,
-                                                        int64_t n, const uint32_t *bsum, uint32_t *pre) {
+                                                        int64_t n, const uint32_t *bsum, uint32_t *pre, bool scanned) {
     grid_dep_wait();
-    __shared__ uint32_t wsum[SCAN_NT / 32];
+    __shared__ uint32_t wsum[SCAN_NT / 32], wbase[SCAN_NT / 32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t before = 0;
+    if (!scanned)
+        for (int i = threadIdx.x; i < (int)blockIdx.x; i += SCAN_NT) before += bsum[i];
+    else if (threadIdx.x == 0)
+        before = bsum[blockIdx.x];
     const int64_t b0 = (int64_t)blockIdx.x * SCAN_CH + (int64_t)threadIdx.x * SCAN_PER;
     uint32_t v[SCAN_PER];
     uint32_t s = 0;
@@ -832,37 +848,23 @@ __global__ void __launch_bounds__(SCAN_NT) k_scan_apply(const __grid_constant__ 
         const uint32_t u = __shfl_up_sync(0xffffffffu, inc, d);
         if (lane >= d) inc += u;
     }
-    if (lane == 31) wsum[wid] = inc;
-    __syncthreads();
-    if (wid == 0) {
-        uint32_t w = lane < SCAN_NT / 32 ? wsum[lane] : 0u, wi = w;
-        for (int d = 1; d < 32; d <<= 1) {
-            const uint32_t u = __shfl_up_sync(0xffffffffu, wi, d);
-            if (lane >= d) wi += u;
-        }
-        if (lane < SCAN_NT / 32) wsum[lane] = wi - w;
+    before = __reduce_add_sync(0xffffffffu, before);
+    if (lane == 31) {
+        wsum[wid] = inc;
+        wbase[wid] = before;
     }
     __syncthreads();
-    uint32_t run = bsum[blockIdx.x] + wsum[wid] + inc - s;
+    uint32_t run = inc - s;
+#pragma unroll
+    for (int w = 0; w < SCAN_NT / 32; ++w) {
+        run += wbase[w];
+        if (w < wid) run += wsum[w];
+    }
 #pragma unroll
     for (int j = 0; j < SCAN_PER; ++j) {
         const int64_t i = b0 + j;
         if (i <= n) pre[i] = run;   // pre[n] = total
         run += v[j];
-    }
-}
-
-// per-lattice: cluster count from the prefix, clear the histogram
-template <int NL>
-__global__ void k_lattice_finish(const __grid_constant__ LatBatch<NL> B, Work W) {
-    grid_dep_wait();
-    const int l = blockIdx.x;
-    if (l >= B.n) return;
-    const LatDev &L = B.lat[l];
-    if (threadIdx.x < 32 && L.hist) L.hist[threadIdx.x] = 0;
-    if (threadIdx.x == 0 && L.ncl) {
-        // uint32 difference: the prefix may wrap over a launch, a lattice's count does not
-        L.ncl[0] = (int64_t)(uint32_t)(W.pre[L.row0 + (int64_t)L.nz * L.ny] - W.pre[L.row0]);
     }
 }
 
@@ -1013,6 +1015,10 @@ k_flatten(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles, uint32
         const int nb = ti.w & 0x7ff, total = (ti.w >> 11) & 0x1fff, lat = NL == 1 ? 0 : ti.w >> 24;
         const LatDev &L = B.lat[lat];
         const int r = tid, ly = r % TY, lz = r / TY;
+        // a lattice's count, with its first tile (a uint32 difference: the prefix may wrap over
+        // a launch, a lattice's count does not)
+        if (tid == 0 && L.ncl && (ti.x | ti.y | ti.z) == 0)
+            L.ncl[0] = (int64_t)(uint32_t)(W.pre[L.row0 + (int64_t)L.nz * L.ny] - W.pre[L.row0]);
         // Rank base of this row: the roots of the lattice's earlier rows, then of this row's
         // earlier segments; carried on while the tiles follow each other along x.
         const int q = (ti.z + lz) * L.ny + (ti.y + ly);
@@ -1581,12 +1587,12 @@ static cudaError_t launch_all(const LatDev *lats, int n, const Plan &P, const Wo
     else launch_dep(k_piece_finalize<NL, false>, gpf, 32 * PF_WARPS, 0, st, B, W, P.ntiles, MB);
     mark(4);
     const int64_t nb = (P.nrows + SCAN_CH) / SCAN_CH;   // covers index nrows (the total)
+    const bool scanned = nb > SCAN_DIRECT;
     launch_dep(k_scan_reduce<NL>, (unsigned)nb, SCAN_NT, 0, st, B, (const uint8_t *)W.cnt, P.nrows, W.bsum);
-    launch_dep(k_scan_blocks, 1u, 1024u, 0, st, W.bsum, nb);
+    if (scanned) launch_dep(k_scan_blocks, 1u, 1024u, 0, st, W.bsum, nb);
     launch_dep(k_scan_apply<NL>, (unsigned)nb, SCAN_NT, 0, st, B, (const uint8_t *)W.cnt, P.nrows,
-               (const uint32_t *)W.bsum, W.pre);
+               (const uint32_t *)W.bsum, W.pre, scanned);
     mark(5);
-    launch_dep(k_lattice_finish<NL>, (unsigned)n, 32u, 0, st, B, W);
     mark(6);
     if constexpr (NL == 1) {
         if (W.roots || W.site_off) launch_dep(k_flatten<TY, TZ, NL, true>, g4, SH::NT, smem4, st, B, W, P.ntiles, span4);

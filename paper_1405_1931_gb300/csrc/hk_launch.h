@@ -36,7 +36,7 @@ constexpr int NUM_PASSES = 7;   // occupancy, tile_label, face_merge, piece_fina
 
 // Byte offsets of the workspace buffers of one launch (every offset 256-byte aligned).
 struct Layout {
-    size_t mask, codes, cnt, pre, bsum, face, tinfo, parent, key, psize, xcol, ovf, rootbits, segpre, votes, ncl, total;
+    size_t mask, codes, cnt, pre, face, tinfo, parent, key, psize, xcol, ovf, rootbits, segpre, votes, ncl, total;
 };
 
 // The workspace of one launch.  votes_cap > 0: also the root bits, the segment prefix
@@ -49,12 +49,10 @@ inline Layout make_layout(const TileInfo &ti, const Plan &P, int64_t votes_cap =
         off += (bytes + 255) & ~(size_t)255;
         return o;
     };
-    const int64_t nb = (P.nrows + 4096) / 4096;   // scan blocks (4096 rows each) covering index nrows
     L.mask = take((size_t)P.ntiles * ti.rows * 4);
     L.codes = take((size_t)P.ntiles * ti.maxruns * 2);
     L.cnt = take((size_t)P.nseg);
     L.pre = take((size_t)(P.nrows + 1) * 4);
-    L.bsum = take((size_t)nb * 4);
     L.face = take((size_t)P.ntiles * ti.face_stride * 2);
     L.tinfo = take((size_t)P.ntiles * 16);
     L.parent = take((size_t)P.piece_cap * 4);
