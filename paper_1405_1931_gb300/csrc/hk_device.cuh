@@ -203,6 +203,13 @@ __device__ __forceinline__ bool occupied(float v, int mode) { return mode ? (v <
 __device__ __forceinline__ uint32_t run_starts(uint32_t m) { return m & ~(m << 1); }
 // the last site of every run: bit x set when x is occupied and x + 1 is not (or x = 31)
 __device__ __forceinline__ uint32_t run_ends(uint32_t m) { return m & ~(m >> 1); }
+// Bits o (a subset of m) spread inside their runs of m: to all higher bits of the run
+// (the carry of m + o runs from each run's lowest bit of o to its end), or to all lower
+// ones (the same on reversed words).
+__device__ __forceinline__ uint32_t fill_up(uint32_t m, uint32_t o) { return (((m + o) ^ m) | o) & m; }
+__device__ __forceinline__ uint32_t fill_down(uint32_t m, uint32_t o) {
+    return __brev(fill_up(__brev(m), __brev(o)));
+}
 // position of the highest set bit of w (of the only one, for an isolated bit: one
 // instruction, where __ffs takes two on the same slow pipe)
 __device__ __forceinline__ int top_bit(uint32_t w) {

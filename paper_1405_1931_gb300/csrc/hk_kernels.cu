@@ -177,6 +177,14 @@ __global__ void __launch_bounds__(256) k_occupancy_tma(const __grid_constant__ T
 
 // --------------------------------------------------------------------------------------
 // K1: tile labelling from the occupancy words (one tile per CTA)
+//
+// Bound by instruction issue (90 % of its rate): 2.2 warp instructions a site at p_c.
+// With most pairs linked or left out instead of united, and with boundary roots listed
+// by a counter instead of two passes and a scan over all runs: 2.11 against 2.38 ms at
+// 1024^3, p_c, 0.83 against 1.06 ms on blocks of 16^3, 0.130 against 0.148 ms on a 512^3
+// bijel.  Where it goes at p_c (cumulative cuts): loads and geometry 0.22 ms, run ids and
+// nodes 0.16, pair words and their scan 0.06, links and lists 0.17, unions 0.30,
+// compression and sizes 0.39, boundary pieces 0.41, row counts 0.04, codes 0.18, faces 0.18.
 // --------------------------------------------------------------------------------------
 template <int TY, int TZ, int CAP, int BL>
 struct LabelSmem {
@@ -187,16 +195,14 @@ struct LabelSmem {
     int aux[CAP];                          // union pair lists; then per root: size + AUX_FACE *
                                            // (runs touching a face); then -1 - k for boundary root k
     uint16_t desc[CAP];                    // per run: DESC_TOUCH | (tile row << 5) | first x
-    uint16_t blist[BL];                    // run ids of the boundary roots, by boundary number
+    uint16_t blist[BL];                    // run id of each boundary root, by its number
     uint32_t nylo[TZ], nyhi[TZ];           // neighbour rows across the y faces, per plane
     uint32_t nzlo[TY], nzhi[TY];           // neighbour rows across the z faces, per row
     uint32_t nxlo[SH::R / 32], nxhi[SH::R / 32];   // neighbour columns across the x faces
     uint32_t xo0[SH::R / 32], xol[SH::R / 32];     // this tile's first and last column
     static_assert(TZ <= 16 && TY <= 32 && SH::R / 32 <= 16 && SH::NT >= 64, "face loads use threads 0..63");
     static_assert(SH::R <= 256 && CAP <= 4096, "desc holds an 8-bit row and run ids fit in 16 bits");
-    uint32_t chunkbal[CAP / 32];           // boundary-root ballot of each chunk of 32 run ids
-    uint32_t chunkint[CAP / 32];           // interior-root ballot of each chunk
-    int chunkpre[CAP / 32];                // boundary roots before each chunk
+    uint32_t rowcnt[SH::R / 4];            // interior roots of each row, a byte each
     int nbnd;                              // boundary roots of the tile
     int warp_tmp[32];
 };
@@ -298,39 +304,42 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
             if ((S.nxlo[r >> 5] >> (r & 31)) & 1u) conn |= 1u;
             if ((S.nxhi[r >> 5] >> (r & 31)) & 1u) conn |= 1u << g.lastX;
             conn &= m;
-            // The run starts whose run holds a connected site, for the whole row at once:
-            // conn is spread towards lower x inside each run by doubling (after the step
-            // of shift s, bit i holds the OR of conn over [i, i + 2s - 1] when m is set
-            // all the way from i; rr marks where m is set over [i, i + s]).
-            uint32_t f = conn, rr = m & (m >> 1);
-            f |= (f >> 1) & rr;
-            rr &= rr >> 1;
-            f |= (f >> 2) & rr;
-            rr &= rr >> 2;
-            f |= (f >> 4) & rr;
-            rr &= rr >> 4;
-            f |= (f >> 8) & rr;
-            rr &= rr >> 8;
-            f |= (f >> 16) & rr;
-            const uint32_t touched = f & rs;
-            uint32_t w = rs;
+            // the run starts whose run holds a connected site, for the whole row at once
+            const uint32_t touched = fill_down(m, conn) & rs;
             int id = rb;
-            while (w) {
-                const int x0 = __ffs(w) - 1;
-                w &= w - 1;
+            for (uint32_t w = rs; w;) {
+                const uint32_t low = w & (0u - w);
+                w ^= low;
                 S.par[id] = id;
-                S.desc[id] = (uint16_t)((((touched >> x0) & 1u) ? DESC_TOUCH : 0) | (r << 5) | x0);
+                S.desc[id] = (uint16_t)(((touched & low) ? DESC_TOUCH : 0) | (r << 5) | top_bit(low));
                 ++id;
             }
         }
         const int ucap = (W.local_cap > 0 && W.local_cap < total) ? W.local_cap : total;   // union retry bound
 
         // y- and z-neighbours: one union per overlapping run pair of rows (y-1, y) and
-        // (z-1, z).  Both pair lists come from one scan of packed counts (each total
-        // is at most 16 * R < 2^16) and normally share one pass of unions, the z pairs
-        // listed first (measured faster than y first).
-        const uint32_t osy = ly > 0 ? run_starts(m & S.m[r - 1]) : 0u;
-        const uint32_t osz = lz > 0 ? run_starts(m & S.m[r - TY]) : 0u;
+        // (z-1, z), that is per segment of their common sites.  Two kinds of pairs need
+        // none.  A run's first pair -- with row y - 1, or with row z - 1 if it meets no run
+        // of row y - 1 -- is written straight into its own node (link): a smaller id, and
+        // the node has no other writer yet, so no find and no atomic.  And a z pair is left
+        // out where it starts at a site x with (x, y-1, z) and (x, y-1, z-1) occupied too:
+        // the two runs are joined through those, by their own y pairs and the z pair of row
+        // y - 1 (or what that one is joined through, down to the tile's first row).
+        // At p_c 0.2 unions a run are left of 0.8, in smooth fields hardly any.
+        // Both lists of the others come from one scan of packed counts (each total is at
+        // most 16 * R < 2^16) and normally share one pass of unions, the z pairs listed
+        // first (measured faster than y first).
+        const uint32_t my = ly > 0 ? S.m[r - 1] : 0u, mz = lz > 0 ? S.m[r - TY] : 0u;
+        const uint32_t oy = m & my, oz = m & mz, uy = fill_up(m, oy);
+        uint32_t osy = run_starts(oy), osz = run_starts(oz);
+        uint32_t link = osy & ~(uy << 1);                      // first y pair of each run
+        osy ^= link;
+        {
+            const uint32_t zlink = osz & ~(fill_up(m, oz) << 1) & ~(uy | fill_down(m, oy));
+            link |= zlink;
+            osz &= ~zlink;
+            if (ly > 0 && lz > 0) osz &= ~(my & S.m[r - TY - 1]);
+        }
         int tot_packed;
         const int packed = block_exscan<NT>(__popc(osy) | (__popc(osz) << 16), S.warp_tmp, tot_packed);
         const int ny_tot = tot_packed & 0xffff, nz_tot = tot_packed >> 16;
@@ -338,14 +347,20 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
             if (tid == 0) W.ovf[atomicAdd(W.novf, 1)] = (int32_t)t;
             continue;
         }
-        auto write_pairs = [&](uint32_t os, int q, int j) {
-            const uint32_t mq = S.m[q];
-            const uint32_t rsq = run_starts(mq);
-            const int rbq = S.rbase[q];
+        // run ids at a site of rows r (rb), r - 1 (rby) and r - TY (rbz): the run starts up to it
+        const uint32_t rsy = run_starts(my), rsz = run_starts(mz);
+        const int rby = ly > 0 ? S.rbase[r - 1] : 0, rbz = lz > 0 ? S.rbase[r - TY] : 0;
+        while (link) {
+            const uint32_t low = link & (0u - link), le = low | (low - 1u);
+            link ^= low;
+            const bool y = (my & low) != 0u;                   // a z link's run meets no run of row y - 1
+            S.par[rb + __popc(rs & le) - 1] = (y ? rby : rbz) + __popc((y ? rsy : rsz) & le) - 1;
+        }
+        auto write_pairs = [&](uint32_t os, uint32_t rsq, int rbq, int j) {
             while (os) {
-                const int x = __ffs(os) - 1;
-                os &= os - 1;
-                S.aux[j++] = (run_of(rb, rs, x) << 16) | run_of(rbq, rsq, x);
+                const uint32_t low = os & (0u - os), le = low | (low - 1u);
+                os ^= low;
+                S.aux[j++] = ((rb + __popc(rs & le) - 1) << 16) | (rbq + __popc(rsq & le) - 1);
             }
         };
         auto union_pairs = [&](int n) {
@@ -355,17 +370,17 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
             }
         };
         if (ny_tot + nz_tot <= CAP) {           // block-uniform
-            if (osz) write_pairs(osz, r - TY, packed >> 16);
-            if (osy) write_pairs(osy, r - 1, nz_tot + (packed & 0xffff));
+            write_pairs(osz, rsz, rbz, packed >> 16);
+            write_pairs(osy, rsy, rby, nz_tot + (packed & 0xffff));
             __syncthreads();
             union_pairs(ny_tot + nz_tot);
             __syncthreads();
         } else {
-            if (osy) write_pairs(osy, r - 1, packed & 0xffff);
+            write_pairs(osy, rsy, rby, packed & 0xffff);
             __syncthreads();
             union_pairs(ny_tot);
             __syncthreads();
-            if (osz) write_pairs(osz, r - TY, packed >> 16);
+            write_pairs(osz, rsz, rbz, packed >> 16);
             __syncthreads();
             union_pairs(nz_tot);
             __syncthreads();
@@ -385,6 +400,8 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
         }
 
         // Sizes accumulate in aux, which held the pair lists until the unions above.
+        if (tid < R / 4) S.rowcnt[tid] = 0u;
+        if (tid == 0) S.nbnd = 0;
         for (int i = 4 * tid; i < total; i += 4 * NT)
             *reinterpret_cast<int4 *>(&S.aux[i]) = make_int4(0, 0, 0, 0);
         __syncthreads();
@@ -395,7 +412,8 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
         // others still search is safe.  A piece is a boundary piece iff its sum reaches
         // AUX_FACE (sizes stay below it).
         for (int i = tid; i < total; i += NT) {
-            const int root = s_find_ro(S.par, i);
+            int root = S.par[i];
+            for (int up = S.par[root]; up != root; up = S.par[root]) root = S.par[up];   // two levels a step
             S.par[i] = root;
             const int d = S.desc[i];
             const int len = run_len(S.m[(d >> 5) & 0xff], d & 31);
@@ -403,62 +421,34 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
         }
         __syncthreads();
 
-        // Number the boundary roots in run order and write their records to the tile's
-        // slice of the piece table.  Chunks of 32 run ids are counted by ballot, the chunk
-        // counts scanned by one warp, and the boundary roots listed by number, so that only
-        // they do the record writes.  Interior roots are kept as a ballot per chunk for the
-        // per-row counts below.
+        // Number the boundary roots (in any order: the number only names the piece) and list
+        // them, so that only they do the record writes; interior roots are counted per row.
         const int base = (int)(t * SH::MAX_BOUNDARY);   // fixed slice of the piece table
         {
-            const int lane = tid & 31, wid = tid >> 5;
-            constexpr int NW = NT / 32;
-            const int nchunks = (total + 31) / 32;
-            for (int c = wid; c < nchunks; c += NW) {
-                const int i = c * 32 + lane;
+            const int lane = tid & 31;
+            for (int i0 = tid - lane; i0 < total; i0 += NT) {
+                const int i = i0 + lane;
                 const bool root = i < total && S.par[i] == i;
                 const bool bnd = root && S.aux[i] >= AUX_FACE;
-                const uint32_t bb = __ballot_sync(0xffffffffu, bnd);
-                const uint32_t bi = __ballot_sync(0xffffffffu, root && !bnd);
-                if (lane == 0) {
-                    S.chunkbal[c] = bb;
-                    S.chunkint[c] = bi;
+                const uint32_t bal = __ballot_sync(0xffffffffu, bnd);
+                if (bal) {
+                    int k0 = 0;
+                    if (lane == 0) k0 = atomicAdd(&S.nbnd, __popc(bal));
+                    const int k = __shfl_sync(0xffffffffu, k0, 0) + __popc(bal & ((1u << lane) - 1u));
+                    if (bnd && k < BL) S.blist[k] = (uint16_t)i;
+                }
+                if (root && !bnd) {
+                    const int row = (S.desc[i] >> 5) & 0xff;
+                    atomicAdd(&S.rowcnt[row >> 2], 1u << (8 * (row & 3)));   // a byte a row: at most 16
                 }
             }
-            __syncthreads();
-            if (wid == 0) {   // at most CAP / 32 <= 128 chunks
-                int carry = 0;
-                for (int c0 = 0; c0 < nchunks; c0 += 32) {
-                    const int c = c0 + lane;
-                    const int v = c < nchunks ? __popc(S.chunkbal[c]) : 0;
-                    int inc = v;
-#pragma unroll
-                    for (int d = 1; d < 32; d <<= 1) {
-                        const int u = __shfl_up_sync(0xffffffffu, inc, d);
-                        if (lane >= d) inc += u;
-                    }
-                    if (c < nchunks) S.chunkpre[c] = carry + inc - v;
-                    carry += __shfl_sync(0xffffffffu, inc, 31);
-                }
-                if (lane == 0) S.nbnd = carry;
-            }
-            __syncthreads();
         }
+        __syncthreads();
         const int nb_ = S.nbnd;
         if (FAST && nb_ > BL) {                 // block-uniform; nothing global written yet
             if (tid == 0) W.ovf[atomicAdd(W.novf, 1)] = (int32_t)t;
             continue;
         }
-        {
-            const int lane = tid & 31, wid = tid >> 5;
-            constexpr int NW = NT / 32;
-            const int nchunks = (total + 31) / 32;
-            for (int c = wid; c < nchunks; c += NW) {
-                const uint32_t bal = S.chunkbal[c];
-                if ((bal >> lane) & 1u)
-                    S.blist[S.chunkpre[c] + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(c * 32 + lane);
-            }
-        }
-        __syncthreads();
         for (int k = tid; k < nb_; k += NT) {
             const int i = S.blist[k];
             const int d = S.desc[i];
@@ -474,24 +464,10 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
                                    nb_ | (total << 11) | (lat << 24));
         __syncthreads();
 
-        // interior roots per row segment (a row's runs span at most two chunks)
-        if (ly <= g.lastY && lz <= g.lastZ) {
-            const int n = __popc(rs);
-            int interior = 0;
-            if (n) {
-                const int a = rb, b = rb + n - 1;             // the row's run ids [a, b]
-                const int ca = a >> 5, cb = b >> 5;
-                const uint32_t lo = S.chunkint[ca] >> (a & 31);
-                if (ca == cb) {
-                    interior = __popc(lo & ((1u << n) - 1u));   // n <= 16
-                } else {
-                    const int nh = (b & 31) + 1;                 // ids of the row in chunk cb
-                    interior = __popc(lo) + __popc(S.chunkint[cb] & ((1u << nh) - 1u));
-                }
-            }
-            const int64_t seg = L.seg0 + ((int64_t)(g.z0 + lz) * L.ny + (g.y0 + ly)) * L.nbx + g.bx;
-            W.cnt[seg] = (uint8_t)interior;
-        }
+        // interior roots per row segment
+        if (ly <= g.lastY && lz <= g.lastZ)
+            W.cnt[L.seg0 + ((int64_t)(g.z0 + lz) * L.ny + (g.y0 + ly)) * L.nbx + g.bx] =
+                reinterpret_cast<const uint8_t *>(S.rowcnt)[r];
 
         // one code per run (CODE_* encoding): aux of the run's root is -1 - k for boundary
         // piece k, else the interior piece's size
