@@ -872,7 +872,9 @@ constexpr int FLAT_ITEMS = 8;
 template <int TY, int TZ>
 struct FlatSmem {
     using SH = TileShape<TY, TZ>;
-    static constexpr int GL = SH::MAX_BOUNDARY < 256 ? SH::MAX_BOUNDARY : 256;   // staged boundary pieces
+    // staged boundary pieces (a tile at p_c has about 124), few enough that six CTAs share an SM
+    // (256 of them and five CTAs: 1.39 against 1.35 ms at 1024^3, p_c)
+    static constexpr int GL = SH::MAX_BOUNDARY < 192 ? SH::MAX_BOUNDARY : 192;
     static constexpr int CC = SH::MR_FAST;                                       // staged run codes
     static_assert(GL % 4 == 0 && CC % 8 == 0 && (SH::MAX_BOUNDARY * 4) % 16 == 0 && (SH::MAXRUNS * 2) % 16 == 0,
                   "bulk copies of whole 16-byte blocks from 16-byte aligned slices");
