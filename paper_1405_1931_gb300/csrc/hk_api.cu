@@ -26,7 +26,7 @@ Work bind_work(char *base, const Layout &Ly, int32_t *status, int64_t piece_cap,
     W.codes = reinterpret_cast<uint16_t *>(base + Ly.codes);
     W.cnt = reinterpret_cast<uint8_t *>(base + Ly.cnt);
     W.pre = reinterpret_cast<uint32_t *>(base + Ly.pre);
-    W.bsum = reinterpret_cast<uint32_t *>(base + Ly.parent);
+    W.bsum = reinterpret_cast<uint32_t *>(base + Ly.face);
     W.face = reinterpret_cast<uint16_t *>(base + Ly.face);
     W.tinfo = reinterpret_cast<int4 *>(base + Ly.tinfo);
     W.parent = reinterpret_cast<int32_t *>(base + Ly.parent);
@@ -35,9 +35,10 @@ Work bind_work(char *base, const Layout &Ly, int32_t *status, int64_t piece_cap,
     W.xcol = reinterpret_cast<uint32_t *>(base + Ly.xcol);
     W.status = status;
     W.ovf = reinterpret_cast<int32_t *>(base + Ly.ovf);
-    W.rootbits = reinterpret_cast<uint32_t *>(base + Ly.rootbits);
-    W.segpre = reinterpret_cast<uint32_t *>(base + Ly.segpre);
-    W.votes = reinterpret_cast<int32_t *>(base + Ly.votes);
+    W.neg = reinterpret_cast<uint32_t *>(base + Ly.neg);
+    W.pos = reinterpret_cast<uint32_t *>(base + Ly.pos);
+    W.pvotes = reinterpret_cast<int32_t *>(base + Ly.pvotes);
+    W.tag = reinterpret_cast<uint32_t *>(base + Ly.tag);
     W.novf = status + 1;
     W.piece_cap = (loop_cap > 0 && loop_cap < piece_cap) ? loop_cap : piece_cap;
     W.local_cap = (loop_cap > 0 && loop_cap < INT32_MAX) ? (int32_t)loop_cap : 0;
@@ -55,8 +56,6 @@ struct hk_ctx {
     size_t ws_bytes = 0;
     void *io = nullptr;       // device buffers of hk_label_host
     size_t io_bytes = 0;
-    void *sbuf = nullptr;     // device buffers of hk_interior_state
-    size_t sbuf_bytes = 0;
     int last_cuda = 0;
     int32_t *dstatus = nullptr;   // device status word (STATUS_* flags), survives workspace growth
     int64_t loop_cap = 0;         // test bound of the capped union-find loops (0: natural bounds)
@@ -284,7 +283,7 @@ int run_small(hk_ctx *ctx, const hk_lattice *lats, int n, cudaStream_t st, bool 
 // (I < -0.5) and, when inside != nullptr, write the interior/exterior tags of its
 // clusters to inside.
 // check_capacity == false: never wait for the counts (the caller compares them).
-// state != nullptr (index fields with inside): also the interior state of every site.
+// state != nullptr (index fields): the interior state of every site, and nothing else.
 int run_lattices(hk_ctx *ctx, const hk_lattice *lats, int n, cudaStream_t st, bool index_field = false,
                  int8_t *inside = nullptr, bool check_capacity = true, int8_t *state = nullptr,
                  int64_t site_off = 0, int32_t *roots = nullptr) {
@@ -350,7 +349,7 @@ int run_lattices(hk_ctx *ctx, const hk_lattice *lats, int n, cudaStream_t st, bo
         Plan P{0, 0, 0, 0};
         for (int i = chunk_start[c]; i < chunk_start[c + 1]; ++i) add_lattice(ti, lats[i].nx, lats[i].ny, lats[i].nz, P);
         P.piece_cap = P.ntiles * ti.max_boundary;
-        need = std::max(need, hk::make_layout(ti, P, inside ? lats[0].sizes_cap : 0).total);
+        need = std::max(need, hk::make_layout(ti, P, inside || state).total);
     }
     int rc = ensure_ws(ctx, need);
     if (rc != HK_OK) return rc;
@@ -387,13 +386,12 @@ int run_lattices(hk_ctx *ctx, const hk_lattice *lats, int n, cudaStream_t st, bo
             add_lattice(ti, l.nx, l.ny, l.nz, P);
         }
         P.piece_cap = P.ntiles * ti.max_boundary;
-        const hk::Layout Ly = hk::make_layout(ti, P, inside ? lats[0].sizes_cap : 0);
+        const hk::Layout Ly = hk::make_layout(ti, P, inside || state);
         char *base = static_cast<char *>(ctx->ws);
         Work W = hk::bind_work(base, Ly, ctx->dstatus, P.piece_cap, ctx->loop_cap);
-        if (!inside) {
-            W.rootbits = nullptr;
-            W.segpre = nullptr;
-            W.votes = nullptr;
+        if (!inside && !state) {
+            W.neg = W.pos = W.tag = nullptr;
+            W.pvotes = nullptr;
         }
         W.site_off = site_off;   // slab calls: one lattice
         W.roots = roots;
@@ -414,12 +412,8 @@ int run_lattices(hk_ctx *ctx, const hk_lattice *lats, int n, cudaStream_t st, bo
         }
         std::vector<hk::PhiTmap> tms(cn);
         for (int i = 0; i < cn; ++i) make_tmap(lats[c0 + i], ctx->ty, ctx->tz, tms[i]);
-        e = hk::launch_label(ctx->ty, ctx->tz, dev.data(), cn, P, W, tms.data(), st, ev, ctx->merge);
+        e = hk::launch_label(ctx->ty, ctx->tz, dev.data(), cn, P, W, tms.data(), st, ev, ctx->merge, state);
         if (e != cudaSuccess) return fail_cuda(ctx, e);
-        if (inside && dev[0].sizes_cap > 0) {
-            e = hk::launch_interior(dev[0], W, st, state);
-            if (e != cudaSuccess) return fail_cuda(ctx, e);
-        }
         if (chunk_check) {
             // the capacity rule needs the counts: wait for this chunk
             any_check = true;
@@ -552,7 +546,6 @@ void hk_destroy(hk_ctx *ctx) {
     cudaSetDevice(ctx->device);
     if (ctx->ws) cudaFree(ctx->ws);
     if (ctx->io) cudaFree(ctx->io);
-    if (ctx->sbuf) cudaFree(ctx->sbuf);
     if (ctx->dstatus) cudaFree(ctx->dstatus);
     if (ctx->dcounts) cudaFree(ctx->dcounts);
     if (ctx->slab_fmap) cudaFree(ctx->slab_fmap);
@@ -621,28 +614,13 @@ int hk_interior_state(hk_ctx *ctx, const float *index, int nx, int ny, int nz, c
     if (N >= MAX_SITES) return HK_ERR_TOO_LARGE;
     cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return fail_cuda(ctx, e);
-    // labels, sizes, histogram, count and tags of the far sites' clusters, in the
-    // context; ceil(N / 2) clusters always fit
-    const int64_t cap = (N + 1) / 2;
-    const size_t o_lab = 0, o_sizes = align256(4 * N), o_hist = o_sizes + align256(8 * cap);
-    const size_t o_ncl = o_hist + 256, o_inside = o_ncl + 256, need = o_inside + align256(cap);
-    if (need > ctx->sbuf_bytes) {
-        if (ctx->sbuf) { cudaDeviceSynchronize(); cudaFree(ctx->sbuf); ctx->sbuf = nullptr; ctx->sbuf_bytes = 0; }
-        if (cudaMalloc(&ctx->sbuf, need) != cudaSuccess) { cudaGetLastError(); return HK_ERR_NOMEM; }
-        ctx->sbuf_bytes = need;
-    }
-    char *b = static_cast<char *>(ctx->sbuf);
     hk_lattice l;
+    std::memset(&l, 0, sizeof(l));
     l.phi = index;
     l.nx = nx; l.ny = ny; l.nz = nz;
     for (int a = 0; a < 3; ++a) l.periodic[a] = periodic[a];
-    l.labels = reinterpret_cast<int32_t *>(b + o_lab);
-    l.sizes = reinterpret_cast<int64_t *>(b + o_sizes);
-    l.sizes_cap = cap;
-    l.hist = reinterpret_cast<int64_t *>(b + o_hist);
-    l.n_clusters = reinterpret_cast<int64_t *>(b + o_ncl);
-    return run_lattices(ctx, &l, 1, static_cast<cudaStream_t>(stream), true, reinterpret_cast<int8_t *>(b + o_inside),
-                        false, state_out);
+    l.labels = reinterpret_cast<int32_t *>(state_out);   // not written as labels: the state is all that comes out
+    return run_lattices(ctx, &l, 1, static_cast<cudaStream_t>(stream), true, nullptr, false, state_out);
 }
 
 int hk_interior_update(const int8_t *state_prev, const float *index, int64_t n_sites, int8_t *state_out,

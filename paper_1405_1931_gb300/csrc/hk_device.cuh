@@ -62,7 +62,7 @@ struct Work {
     uint16_t *codes;    // [ntiles * MAXRUNS] one code per run (CODE_* above)
     uint8_t *cnt;       // [nseg] cluster roots per segment (row-major segment order; <= 16)
     uint32_t *pre;      // [nrows + 1] exclusive prefix of the roots per lattice row
-    uint32_t *bsum;     // [nblocks] scan block sums (in parent's space, which is free by then)
+    uint32_t *bsum;     // [nblocks] scan block sums (in face's space, which is free by then)
     uint16_t *face;     // [ntiles * face_stride] per-face lists of boundary-piece numbers
     int4 *tinfo;        // [ntiles] each tile's first site (x, y, z) and its counts: boundary pieces
                         // (bits 0-10), runs (bits 11-23), lattice of the launch (bits 24-29)
@@ -75,9 +75,14 @@ struct Work {
     uint32_t *xcol;     // [ntiles * 2 * R/32] occupancy of each tile's first (x = 0) and last
                         // (x = lastX) column, one bit per tile row
     int32_t *status;    // [1] device-side error flags (STATUS_*), owned by the context
-    uint32_t *rootbits; // [nseg] cluster-root run starts of each row segment (index fields only)
-    uint32_t *segpre;   // [nseg] clusters ranked before each row segment (index fields only)
-    int32_t *votes;     // [sizes_cap] sign votes per cluster (index fields only)
+    // interior/exterior identification (index fields whose tags or states are wanted, else
+    // null): signs of the near sites, one bit a site laid out like mask, and per piece the
+    // votes of its sites (after piece_finalize a root's are its cluster's), for interior
+    // pieces per run the tag that the votes give (two words per 32 runs: bit set where
+    // interior, bit set where undetermined)
+    uint32_t *neg, *pos;
+    int32_t *pvotes;    // [piece_cap]
+    uint32_t *tag;      // [ntiles * MAXRUNS / 16]
     int32_t *ovf;       // [ntiles] tiles with more runs than the fast tile pass holds
     int32_t *novf;      // [1] entries of ovf (reset by the occupancy pass of every call)
     int64_t piece_cap;  // bound of every global union-find loop: the entries of parent/key/psize

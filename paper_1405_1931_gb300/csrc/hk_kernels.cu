@@ -25,6 +25,12 @@
 
 namespace hk {
 
+// A site near a membrane (Sec. 6, step 2) votes with the sign of its index value: bit q
+// when it is negative, bit 16 + q when positive (not for 0, NaN and the far sites).
+__device__ __forceinline__ uint32_t near_bits(float v, int q) {
+    return (v >= -0.5f && v < 0.0f ? 1u << q : 0u) | (v > 0.0f ? 0x10000u << q : 0u);
+}
+
 // --------------------------------------------------------------------------------------
 // K0: occupancy.  One warp per tile streams phi row by row (one coalesced 128-byte
 // load per row, 16 rows in flight per warp) and keeps phi > 0 (Sec. 2) as one
@@ -52,8 +58,8 @@ __global__ void __launch_bounds__(256, 4) k_occupancy(const __grid_constant__ La
     const bool vec = g.lastX == TX - 1 && (L.nx & 3) == 0 && (reinterpret_cast<uintptr_t>(L.phi) & 15) == 0;
     const int x4 = (lane & 7) * 4;
     const float *base4 = L.phi + (int64_t)g.z0 * sxy + (int64_t)g.y0 * L.nx + g.x0 + x4;
-    for (int r0 = 0; r0 < R; r0 += 32) {        // lane j keeps the word of row r0 + j
-        uint32_t mine = 0;
+    for (int r0 = 0; r0 < R; r0 += 32) {        // lane j keeps the words of row r0 + j
+        uint32_t mine = 0, neg = 0, pos = 0;
         if (vec) {
             float4 v[8];
 #pragma unroll
@@ -73,6 +79,19 @@ __global__ void __launch_bounds__(256, 4) k_occupancy(const __grid_constant__ La
                 w |= __shfl_xor_sync(0xffffffffu, w, 4);
                 const uint32_t wq = __shfl_sync(0xffffffffu, w, (lane & 3) * 8);   // row r0 + 4 q + (lane & 3)
                 if ((lane >> 2) == q) mine = wq;
+                if (W.neg) {                           // uniform: signs of the near sites
+                    uint32_t n = (near_bits(v[q].x, 0) | near_bits(v[q].y, 1) | near_bits(v[q].z, 2) | near_bits(v[q].w, 3));
+                    uint32_t ps = (n >> 16) << x4;
+                    n = (n & 0xffffu) << x4;
+#pragma unroll
+                    for (int d = 1; d < 8; d <<= 1) {
+                        n |= __shfl_xor_sync(0xffffffffu, n, d);
+                        ps |= __shfl_xor_sync(0xffffffffu, ps, d);
+                    }
+                    const uint32_t nq = __shfl_sync(0xffffffffu, n, (lane & 3) * 8);
+                    const uint32_t pq = __shfl_sync(0xffffffffu, ps, (lane & 3) * 8);
+                    if ((lane >> 2) == q) { neg = nq; pos = pq; }
+                }
             }
         } else {
 #pragma unroll
@@ -88,10 +107,19 @@ __global__ void __launch_bounds__(256, 4) k_occupancy(const __grid_constant__ La
                 for (int u = 0; u < U; ++u) {
                     const uint32_t w = __ballot_sync(0xffffffffu, occupied(v[u], L.occ_mode));
                     if (lane == u0 + u) mine = w;
+                    if (W.neg) {
+                        const uint32_t n = near_bits(v[u], 0);
+                        const uint32_t wn = __ballot_sync(0xffffffffu, n & 1u), wp = __ballot_sync(0xffffffffu, n >> 16);
+                        if (lane == u0 + u) { neg = wn; pos = wp; }
+                    }
                 }
             }
         }
         out[r0 + lane] = mine;
+        if (W.neg) {
+            W.neg[t * R + r0 + lane] = neg;
+            W.pos[t * R + r0 + lane] = pos;
+        }
         // first and last column of the tile, one bit per row (faces along x)
         const uint32_t c0 = __ballot_sync(0xffffffffu, mine & 1u);
         const uint32_t cl = __ballot_sync(0xffffffffu, (mine >> g.lastX) & 1u);
@@ -163,6 +191,17 @@ __global__ void __launch_bounds__(256) k_occupancy_tma(const __grid_constant__ T
                 if (lane == j) mine = w;
             }
             W.mask[t * R + r0 + lane] = mine;
+            if (W.neg) {                               // uniform: signs of the near sites
+                uint32_t neg = 0, pos = 0;
+#pragma unroll 8
+                for (int j = 0; j < 32; ++j) {
+                    const uint32_t n = near_bits(S.buf[s][(r0 + j) * 32 + lane], 0);
+                    const uint32_t wn = __ballot_sync(0xffffffffu, n & 1u), wp = __ballot_sync(0xffffffffu, n >> 16);
+                    if (lane == j) { neg = wn; pos = wp; }
+                }
+                W.neg[t * R + r0 + lane] = neg;
+                W.pos[t * R + r0 + lane] = pos;
+            }
             const uint32_t c0 = __ballot_sync(0xffffffffu, mine & 1u);
             const uint32_t cl = __ballot_sync(0xffffffffu, (mine >> lastX) & 1u);
             if (lane == 0) {
@@ -186,13 +225,13 @@ __global__ void __launch_bounds__(256) k_occupancy_tma(const __grid_constant__ T
 // nodes 0.16, pair words and their scan 0.06, links and lists 0.17, unions 0.30,
 // compression and sizes 0.39, boundary pieces 0.41, row counts 0.04, codes 0.18, faces 0.18.
 // --------------------------------------------------------------------------------------
-template <int TY, int TZ, int CAP, int BL>
+template <int TY, int TZ, int CAP, int BL, bool INDEX>
 struct LabelSmem {
     using SH = TileShape<TY, TZ>;
     uint32_t m[SH::R];                     // occupancy word of each row
     uint16_t rbase[SH::R];                 // first run id of each row
     int par[CAP];                          // union-find over run ids; after compression: the root
-    int aux[CAP];                          // union pair lists; then per root: size + AUX_FACE *
+    alignas(16) int aux[CAP];              // union pair lists; then per root: size + AUX_FACE *
                                            // (runs touching a face); then -1 - k for boundary root k
     uint16_t desc[CAP];                    // per run: DESC_TOUCH | (tile row << 5) | first x
     uint16_t blist[BL];                    // run id of each boundary root, by its number
@@ -205,6 +244,8 @@ struct LabelSmem {
     uint32_t rowcnt[SH::R / 4];            // interior roots of each row, a byte each
     int nbnd;                              // boundary roots of the tile
     int warp_tmp[32];
+    uint32_t neg[INDEX ? SH::R : 1], pos[INDEX ? SH::R : 1];   // signs of the near sites of each row
+    int votes[INDEX ? CAP : 1];            // per root: the votes of its piece's sites
 };
 
 constexpr int AUX_FACE = 1 << 14;   // > any piece size (a tile has at most 8192 sites)
@@ -224,15 +265,16 @@ struct LabelCfg {
 // FAST: tiles t = blockIdx.x, blockIdx.x + gridDim.x, ... below ntiles; a tile with
 // more than MR_FAST runs or union pairs of one kind is appended to W.ovf instead.
 // !FAST: the tiles listed in W.ovf, with room for every tile.
-template <int TY, int TZ, int NL, bool FAST>
-__global__ void __launch_bounds__(TY * TZ, (LabelCfg<TY, TZ, FAST>::BLOCKS))
+// INDEX: an index field whose clusters' votes are wanted (Sec. 6, step 5; one lattice).
+template <int TY, int TZ, int NL, bool FAST, bool INDEX>
+__global__ void __launch_bounds__(TY * TZ, (LabelCfg<TY, TZ, FAST && !INDEX>::BLOCKS))
 k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
     grid_dep_wait();
     using SH = TileShape<TY, TZ>;
     constexpr int R = SH::R, NT = SH::NT, MR = SH::MAXRUNS, CAP = LabelCfg<TY, TZ, FAST>::CAP;
     constexpr int BL = LabelCfg<TY, TZ, FAST>::BL;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    LabelSmem<TY, TZ, CAP, BL> &S = *reinterpret_cast<LabelSmem<TY, TZ, CAP, BL> *>(smem_raw);
+    LabelSmem<TY, TZ, CAP, BL, INDEX> &S = *reinterpret_cast<LabelSmem<TY, TZ, CAP, BL, INDEX> *>(smem_raw);
     const int tid = threadIdx.x;
     const int64_t nwork = FAST ? ntiles : (int64_t)*reinterpret_cast<volatile int32_t *>(W.novf);
 
@@ -245,6 +287,10 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
         const int r = tid, ly = r % TY, lz = r / TY;
         const uint32_t m = W.mask[t * R + r];
         S.m[r] = m;
+        if (INDEX) {
+            S.neg[r] = W.neg[t * R + r];
+            S.pos[r] = W.pos[t * R + r];
+        }
         const uint32_t rs = run_starts(m);
         {
             const uint32_t c0 = __ballot_sync(0xffffffffu, m & 1u);
@@ -404,6 +450,8 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
         if (tid == 0) S.nbnd = 0;
         for (int i = 4 * tid; i < total; i += 4 * NT)
             *reinterpret_cast<int4 *>(&S.aux[i]) = make_int4(0, 0, 0, 0);
+        if (INDEX)
+            for (int i = tid; i < total; i += NT) S.votes[i] = 0;
         __syncthreads();
 
         // Compression and piece sizes, one run id per thread: par[i] = root (the piece's
@@ -420,6 +468,56 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
             atomicAdd(&S.aux[root], len + ((d & DESC_TOUCH) ? AUX_FACE : 0));
         }
         __syncthreads();
+
+        // Votes (Sec. 6, step 5): every face-neighbour pair of a cluster site and a near site
+        // adds the near site's sign to the cluster.  Per row, the signs of the six neighbours
+        // of its sites are words like its own (a row of the tile, of the tile across a face
+        // or across a periodic edge, or its own word moved by one along x), so a run's votes
+        // are counts of bits; rows away from every membrane have none.
+        if (INDEX && m) {
+            const int64_t plane = (int64_t)L.nbx * L.nby;
+            auto row_of = [&](const uint32_t *sw, const uint32_t *gw, int axis, bool hi) -> uint32_t {
+                const int c = axis == 1 ? ly : lz, last = axis == 1 ? g.lastY : g.lastZ, step = axis == 1 ? 1 : TY;
+                if (hi ? c < last : c > 0) return sw[hi ? r + step : r - step];
+                const bool ext = axis == 1 ? (hi ? g.extYhi : g.extYlo) : (hi ? g.extZhi : g.extZlo);
+                if (!ext) return (axis == 1 ? g.wrapY : g.wrapZ) ? sw[hi ? r - c * step : r + last * step] : 0u;
+                const int b = axis == 1 ? g.by : g.bz, nb = axis == 1 ? L.nby : L.nbz, len = axis == 1 ? L.ny : L.nz;
+                const int span = axis == 1 ? TY : TZ;
+                const int nb_tile = hi ? (b < nb - 1 ? b + 1 : 0) : (b > 0 ? b - 1 : nb - 1);
+                const int nc = hi ? 0 : min(span, len - nb_tile * span) - 1;
+                return gw[(t + (nb_tile - b) * (axis == 1 ? (int64_t)L.nbx : plane)) * R + r + (nc - c) * step];
+            };
+            auto along_x = [&](const uint32_t *sw, const uint32_t *gw, bool hi) -> uint32_t {
+                const uint32_t w = sw[r];
+                uint32_t edge = 0;                             // the neighbour of the tile's first / last column
+                if (hi) {
+                    if (g.extXhi) edge = gw[(g.bx < L.nbx - 1 ? t + 1 : t - (L.nbx - 1)) * R + r] & 1u;
+                    else if (g.wrapX) edge = w & 1u;
+                    return (w >> 1) | (edge << g.lastX);
+                }
+                if (g.extXlo) edge = gw[(g.bx > 0 ? t - 1 : t + (L.nbx - 1)) * R + r] >> (g.bx > 0 ? TX - 1 : (L.nx - 1) % TX);
+                else if (g.wrapX) edge = w >> g.lastX;
+                return (w << 1) | (edge & 1u);
+            };
+            uint32_t nw[6], pw[6], any = 0;
+#pragma unroll
+            for (int d = 0; d < 6; ++d) {
+                nw[d] = m & (d < 2 ? along_x(S.neg, W.neg, d & 1) : row_of(S.neg, W.neg, d >> 1, d & 1));
+                pw[d] = m & (d < 2 ? along_x(S.pos, W.pos, d & 1) : row_of(S.pos, W.pos, d >> 1, d & 1));
+                any |= nw[d] | pw[d];
+            }
+            int id = rb;
+            for (uint32_t w = any ? rs : 0u; w; ++id) {
+                const uint32_t low = w & (0u - w), run = fill_up(m, low);
+                w ^= low;
+                if (!(any & run)) continue;
+                int v = 0;
+#pragma unroll
+                for (int d = 0; d < 6; ++d) v += __popc(pw[d] & run) - __popc(nw[d] & run);
+                if (v) atomicAdd(&S.votes[S.par[id]], v);
+            }
+        }
+        if (INDEX) __syncthreads();
 
         // Number the boundary roots (in any order: the number only names the piece) and list
         // them, so that only they do the record writes; interior roots are counted per row.
@@ -457,6 +555,7 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
             W.parent[pid] = pid;
             W.key[pid] = ((g.z0 + row / TY) * L.ny + (g.y0 + row % TY)) * L.nx + g.x0 + (d & 31);
             W.psize[pid] = S.aux[i] & (AUX_FACE - 1);
+            if (INDEX) W.pvotes[pid] = S.votes[i];
             S.aux[i] = -1 - k;                   // from here on: boundary root k
         }
         if (tid == 0)
@@ -481,6 +580,19 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
             else
                 c = a < 0 ? (uint16_t)(CODE_BOUNDARY | (-1 - a)) : (uint16_t)(S.desc[v] & (DESC_TOUCH - 1));
             C[i] = c;
+        }
+
+        if (INDEX) {                              // the tag of each run's piece, as if it were interior
+            const int lane = tid & 31;
+            uint32_t *T = W.tag + t * (MR / 16);
+            for (int i0 = tid - lane; i0 < total; i0 += NT) {
+                const int v = i0 + lane < total ? S.votes[S.par[i0 + lane]] : 1;
+                const uint32_t in = __ballot_sync(0xffffffffu, v < 0), tie = __ballot_sync(0xffffffffu, v == 0);
+                if (lane == 0) {
+                    T[i0 >> 4] = in;
+                    T[(i0 >> 4) + 1] = tie;
+                }
+            }
         }
 
         // Face lists.  A face site is connected when it and its neighbour across the
@@ -647,12 +759,12 @@ __global__ void __launch_bounds__(32 * PF_WARPS)
 k_piece_finalize(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles, int max_boundary) {
     grid_dep_wait();
     __shared__ int hot_target[PF_WARPS];   // per warp: the cluster root its pieces fed most, and the sum
-    __shared__ int hot_sum[PF_WARPS];
+    __shared__ int hot_sum[PF_WARPS], hot_votes[PF_WARPS];
     const int64_t t = (int64_t)blockIdx.x * PF_WARPS + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     // The root that collects most sizes (the percolating cluster's, above all) is added
     // once per warp and then once per CTA; other roots once per group of lanes.
-    int hot = -1, hot_acc = 0;
+    int hot = -1, hot_acc = 0, hot_vacc = 0;
     const int nbnd = t < ntiles ? W.tinfo[t].w & 0x7ff : 0;
     if (nbnd > 0) {
         const LatDev &L = B.lat[(NL == 1) ? 0 : find_lattice(B.lat, B.n, t)];
@@ -660,12 +772,13 @@ k_piece_finalize(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles,
             const int j = j0 + lane;
             const bool valid = j < nbnd;
             const int pid = (int)t * max_boundary + j;
-            int root = -1, add = 0;
+            int root = -1, add = 0, vadd = 0;
             if (valid) {
                 root = g_find_ro(W.parent, pid, W.piece_cap, W.status);
                 if (root != pid) {
                     __stcg(W.parent + pid, root);
                     add = W.psize[pid];
+                    if (W.pvotes) vadd = W.pvotes[pid];     // votes of an index field add up like sizes
                     // from here on key[pid] is the cluster's label and psize[pid] < 0 marks a
                     // non-root; only roots' keys are read by other threads, and a root's key
                     // never changes
@@ -683,6 +796,7 @@ k_piece_finalize(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles,
             const int target = (valid && root != pid) ? root : -1;
             const unsigned peers = __match_any_sync(0xffffffffu, target);
             const int sum = (int)__reduce_add_sync(peers, (unsigned)add);
+            const int vsum = W.pvotes ? (int)__reduce_add_sync(peers, (unsigned)vadd) : 0;
             const bool leader = target >= 0 && lane == __ffs(peers) - 1;
             if (HOT && hot < 0) {   // warp-uniform: the first chunk names the warp's hot root (its largest group)
                 const unsigned key = leader ? ((unsigned)__popc(peers) << 5) | (unsigned)lane : 0u;
@@ -690,29 +804,38 @@ k_piece_finalize(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles,
                 if (best) hot = __shfl_sync(0xffffffffu, target, (int)(best & 31u));
             }
             if (leader) {
-                if (target == hot) hot_acc += sum;
-                else atomicAdd(W.psize + target, sum);
+                if (target == hot) {
+                    hot_acc += sum;
+                    hot_vacc += vsum;
+                } else {
+                    atomicAdd(W.psize + target, sum);
+                    if (vsum) atomicAdd(W.pvotes + target, vsum);
+                }
             }
         }
     }
     if (!HOT) return;
     hot_acc = (int)__reduce_add_sync(0xffffffffu, (unsigned)hot_acc);
+    if (W.pvotes) hot_vacc = (int)__reduce_add_sync(0xffffffffu, (unsigned)hot_vacc);
     if (lane == 0) {
         hot_target[wid] = hot;
         hot_sum[wid] = hot_acc;
+        hot_votes[wid] = hot_vacc;
     }
     __syncthreads();
     if (threadIdx.x < PF_WARPS) {   // one add per distinct hot root of the CTA
         const int h = hot_target[threadIdx.x];
         if (h >= 0) {
             bool first = true;
-            int s = 0;
+            int s = 0, v = 0;
             for (int w = 0; w < PF_WARPS; ++w)
                 if (hot_target[w] == h) {
                     if (w < (int)threadIdx.x) first = false;
                     s += hot_sum[w];
+                    v += hot_votes[w];
                 }
             if (first) atomicAdd(W.psize + h, s);
+            if (first && v) atomicAdd(W.pvotes + h, v);
         }
     }
 }
@@ -1073,16 +1196,22 @@ k_flatten(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles, uint32
         uint32_t bits = 0;                             // the row's runs are bits 0 .. n - 1 (n <= 16)
         if (n) bits = __funnelshift_r(S.rootbal[rb >> 5], S.rootbal[(rb >> 5) + 1], (uint32_t)rb & 31u) &
                       ((1u << n) - 1u);
-        if (L.inside) {                                // index fields: ranks of any root, later
-            uint32_t rootbits = 0;                     // first sites of cluster roots in this row
-            for (uint32_t w = bits; w; w &= w - 1u) rootbits |= 1u << (S.lab[rb + __ffs(w) - 1] - site_row);
-            if (valid_row) W.rootbits[L.seg0 + (int64_t)q * L.nbx + ti.x / TX] = rootbits;
-        }
         // Sizes wait in shared memory until their 32-byte sector is full (a row has fewer roots
         // in a tile than that; the next tile along x brings the rest): stores of single
         // sizes left part-written sectors that cost flatten 0.3 to 0.45 ms at 1024^3, p_c.
         const uint32_t cap = (uint32_t)min(L.sizes_cap, (int64_t)INT32_MAX);   // ranks stay below 2^30
         const uint32_t place = (uint32_t)(reinterpret_cast<uintptr_t>(L.sizes) >> 3);
+        if (L.inside) {                                // index fields: the tags, in rank order like the sizes
+            uint32_t k = rank;
+            for (uint32_t w = bits; w && k < cap; w &= w - 1u, ++k) {
+                const int id = rb + __ffs(w) - 1;
+                const int c = id < CC ? (int)S.codes[id] : (int)__ldg(C + id);
+                const uint32_t *T = W.tag + (size_t)t * (MR / 16) + 2 * (id >> 5);
+                const int v = (c & CODE_BOUNDARY) ? W.pvotes[(size_t)t * MB + (c & CODE_LOW)]
+                            : (T[0] >> (id & 31)) & 1u ? -1 : (T[1] >> (id & 31)) & 1u ? 0 : 1;
+                L.inside[k] = (int8_t)(v < 0 ? 1 : (v > 0 ? 0 : -1));
+            }
+        }
         auto flush = [&](bool all) {                   // the full sectors among ranks lo .. rank - 1, or all
             while (lo < rank) {
                 const uint32_t e = lo + 4u - ((lo + place) & 3u);   // the first rank of the next sector
@@ -1183,166 +1312,85 @@ k_flatten(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles, uint32
 }
 
 // --------------------------------------------------------------------------------------
-// Interior/exterior identification (Sec. 6, step 5) for an index field labelled with
-// occ_mode 1: every face pair (cluster site, near site) votes with the sign of I at
-// the near site; a cluster with more negative votes is interior.  One lattice.
+// Interior state of every site of an index field (Sec. 6: 1 far inside, 0 far outside): a
+// far site (I < -0.5) takes the tag that its cluster's votes give (-1 for a tie), a near
+// site the side its value names (step 2: -d inside, +d outside), 1 for I < 0 and 0
+// otherwise.  Like flatten it decodes the runs of each tile, but it needs neither ranks
+// nor labels: it reads the words and codes and writes a byte a site.  One tile per CTA,
+// one row per thread.
 // --------------------------------------------------------------------------------------
-// Clusters ranked before each row segment of an index field: the roots of the
-// lattice's earlier rows and of the row's earlier segments.  One thread per row.
-__global__ void __launch_bounds__(256) k_segpre(const LatDev L, Work W) {
-    const int64_t rows = (int64_t)L.ny * L.nz;
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < rows; q += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t rowseg = L.seg0 + q * L.nbx;
-        uint32_t acc = W.pre[L.row0 + q] - W.pre[L.row0];
-        for (int b = 0; b < L.nbx; ++b) {
-            W.segpre[rowseg + b] = acc;
-            acc += W.cnt[rowseg + b];
-        }
-    }
-}
-
-// Rank (compacted id - 1) of the cluster whose first site is `lab`: the clusters
-// ranked before its segment and the roots of its segment before it.
-__device__ __forceinline__ int64_t rank_of_root(const LatDev &L, const Work &W, int lab) {
-    const int q = lab / L.nx, x = lab - q * L.nx;
-    const int64_t seg = L.seg0 + (int64_t)q * L.nbx + (x >> 5);
-    return (int64_t)W.segpre[seg] + __popc(W.rootbits[seg] & ((1u << (x & 31)) - 1u));
-}
-
-__global__ void __launch_bounds__(256) k_votes_clear(const LatDev L, Work W) {
-    const int64_t n = *L.ncl < L.sizes_cap ? *L.ncl : L.sizes_cap;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
-        W.votes[k] = 0;
-}
-
-// Votes into the first VOTE_SMEM ranks are summed per CTA in shared memory and
-// added to the global counters once per CTA (a few clusters, such as the exterior
-// fluid, collect most votes); higher ranks go straight to global memory.
-constexpr int VOTE_SMEM = 1024;
-
-// The votes of near site s (value v): one per face neighbour that is a cluster site.
-__device__ __forceinline__ void vote_site(const LatDev &L, const Work &W, int64_t s, float v, int *sv) {
-    if (!(v >= -0.5f)) return;                 // a cluster site (or NaN): not a near site
-    const int sign = v < 0.0f ? -1 : (v > 0.0f ? 1 : 0);
-    if (sign == 0) return;
-    const int dims[3] = {L.nx, L.ny, L.nz};
-    const int x = (int)(s % L.nx);
-    const int64_t q = s / L.nx;
-    const int y = (int)(q % L.ny), z = (int)(q / L.ny);
+template <int TY, int TZ>
+__global__ void __launch_bounds__(TY * TZ) k_state(const LatDev L, Work W, int8_t *state, bool vec) {
+    grid_dep_wait();
+    using SH = TileShape<TY, TZ>;
+    constexpr int R = SH::R, NT = SH::NT, NW = NT / 32, MR = SH::MAXRUNS, MB = SH::MAX_BOUNDARY;
+    __shared__ int8_t ptag[MB];                        // tag of each boundary piece's cluster
+    __shared__ uint2 row[R];                           // bits of the states 1 and -1 of each row
+    __shared__ int warp_tmp[NW];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int64_t t = blockIdx.x;
+    const int4 ti = W.tinfo[t];
+    const int nb = ti.w & 0x7ff;
+    const uint32_t m = W.mask[t * R + tid], near_in = W.neg[t * R + tid];
+    const uint32_t rs = run_starts(m);
+    int inc = __popc(rs);
 #pragma unroll
-    for (int dir = 0; dir < 6; ++dir) {
-        const int axis = dir >> 1;
-        int c[3] = {x, y, z};
-        c[axis] += (dir & 1) ? 1 : -1;
-        if (c[axis] < 0 || c[axis] >= dims[axis]) {
-            if (!L.per[axis]) continue;
-            c[axis] = c[axis] < 0 ? dims[axis] - 1 : 0;
-        }
-        const int lab = L.labels[c[0] + (int64_t)L.nx * (c[1] + (int64_t)L.ny * c[2])];
-        if (lab < 0) continue;
-        const int64_t k = rank_of_root(L, W, lab);
-        if (k >= L.sizes_cap) continue;
-        if (k < VOTE_SMEM) atomicAdd(&sv[k], sign);
-        else atomicAdd(W.votes + k, sign);
+    for (int d = 1; d < 32; d <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, inc, d);
+        if (lane >= d) inc += u;
     }
-}
-
-__global__ void __launch_bounds__(256) k_votes(const LatDev L, Work W) {
-    __shared__ int sv[VOTE_SMEM];
-    for (int i = threadIdx.x; i < VOTE_SMEM; i += blockDim.x) sv[i] = 0;
+    if (lane == 31) warp_tmp[wid] = inc;
+    for (int k = tid; k < nb; k += NT) {
+        const int v = W.pvotes[W.parent[t * MB + k]];  // piece_finalize left every piece at its root
+        ptag[k] = (int8_t)(v < 0 ? 1 : (v > 0 ? 0 : -1));
+    }
     __syncthreads();
-    const int64_t N = (int64_t)L.nx * L.ny * L.nz;
-    for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < N; s += (int64_t)gridDim.x * blockDim.x)
-        vote_site(L, W, s, L.phi[s], sv);
-    __syncthreads();
-    for (int i = threadIdx.x; i < VOTE_SMEM; i += blockDim.x)
-        if (sv[i]) atomicAdd(W.votes + i, sv[i]);
-}
-
-__global__ void __launch_bounds__(256) k_inside(const LatDev L, Work W) {
-    const int64_t n = *L.ncl < L.sizes_cap ? *L.ncl : L.sizes_cap;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-        const int v = W.votes[k];
-        L.inside[k] = (int8_t)(v < 0 ? 1 : (v > 0 ? 0 : -1));
-    }
-}
-
-// Interior state of every site (Sec. 6: 1 far inside, 0 far outside): a far site
-// (I < -0.5) takes its cluster's tag, a near site the side its value names (step 2:
-// -d inside, +d outside), 1 for I < 0 and 0 otherwise.  Two passes: each cluster's
-// first site (labels[s] == s) gets the tag of its rank, then every far site copies the
-// tag from its label's site.  Near sites are never a cluster's first site, so the
-// second pass only rewrites first sites with the value they hold.
-__device__ __forceinline__ void state_root(const LatDev &L, const Work &W, int8_t *state, int64_t s, int lab) {
-    if (lab != s) return;
-    const int64_t k = rank_of_root(L, W, (int)s);
-    state[s] = k < L.sizes_cap ? L.inside[k] : (int8_t)-1;
-}
-
-// vec: labels 16-byte aligned, 4 sites at a time
-__global__ void __launch_bounds__(256) k_state_roots(const LatDev L, Work W, int8_t *state, bool vec) {
-    const int64_t N = (int64_t)L.nx * L.ny * L.nz;
-    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
-    int64_t done = 0;
-    if (vec) {
-        for (int64_t i = t0; i < N / 4; i += stride) {
-            const int4 lb = __ldcs(reinterpret_cast<const int4 *>(L.labels) + i);
-            state_root(L, W, state, 4 * i, lb.x);
-            state_root(L, W, state, 4 * i + 1, lb.y);
-            state_root(L, W, state, 4 * i + 2, lb.z);
-            state_root(L, W, state, 4 * i + 3, lb.w);
-        }
-        done = N / 4 * 4;
-    }
-    for (int64_t s = done + t0; s < N; s += stride) state_root(L, W, state, s, L.labels[s]);
-}
-
-__device__ __forceinline__ uint32_t state_byte(const int8_t *state, float v, int lab) {
-    if (v < -0.5f) return (uint32_t)(uint8_t)state[lab];
-    return v < 0.0f ? 1u : 0u;
-}
-
-// vec: phi, labels and state 16-byte aligned, 16 sites at a time (one 16-byte store)
-__global__ void __launch_bounds__(256) k_state(const LatDev L, int8_t *state, bool vec) {
-    const int64_t N = (int64_t)L.nx * L.ny * L.nz;
-    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
-    int64_t done = 0;
-    if (vec) {
-        for (int64_t i = t0; i < N / 16; i += stride) {
-            uint32_t w[4];
+    int id = inc - __popc(rs);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const float4 v = __ldcs(reinterpret_cast<const float4 *>(L.phi) + 4 * i + q);
-                const int4 lb = __ldcs(reinterpret_cast<const int4 *>(L.labels) + 4 * i + q);
-                w[q] = state_byte(state, v.x, lb.x) | (state_byte(state, v.y, lb.y) << 8) |
-                       (state_byte(state, v.z, lb.z) << 16) | (state_byte(state, v.w, lb.w) << 24);
-            }
-            reinterpret_cast<int4 *>(state)[i] = make_int4((int)w[0], (int)w[1], (int)w[2], (int)w[3]);
+    for (int w = 0; w < NW; ++w)
+        if (w < wid) id += warp_tmp[w];
+    uint32_t ones = near_in, ties = 0;
+    for (uint32_t w = rs; w; ++id) {
+        const uint32_t low = w & (0u - w), run = fill_up(m, low);
+        w ^= low;
+        const int c = __ldg(W.codes + t * MR + id);
+        int tag;
+        if (c & CODE_BOUNDARY) {
+            tag = ptag[c & CODE_LOW];
+        } else {
+            const uint32_t *T = W.tag + t * (MR / 16) + 2 * (id >> 5);
+            tag = (__ldg(T) >> (id & 31)) & 1u ? 1 : ((__ldg(T + 1) >> (id & 31)) & 1u ? -1 : 0);
         }
-        done = N / 16 * 16;
+        if (tag > 0) ones |= run;
+        if (tag < 0) ties |= run;
     }
-    for (int64_t s = done + t0; s < N; s += stride) state[s] = (int8_t)state_byte(state, L.phi[s], L.labels[s]);
-}
-
-cudaError_t launch_interior(const LatDev &L, const Work &W, cudaStream_t st, int8_t *state) {
-    int dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t N = (int64_t)L.nx * L.ny * L.nz;
-    int64_t gv = (N + 255) / 256;
-    if (gv > (int64_t)nsm * 16) gv = (int64_t)nsm * 16;
-    const unsigned gc = (unsigned)(nsm > 0 ? nsm * 4 : 1);
-    k_votes_clear<<<gc, 256, 0, st>>>(L, W);
-    auto a16 = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
-    const int64_t rows = (int64_t)L.ny * L.nz;
-    k_segpre<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(L, W);
-    k_votes<<<(unsigned)(gv > 0 ? gv : 1), 256, 0, st>>>(L, W);
-    k_inside<<<gc, 256, 0, st>>>(L, W);
-    if (state) {
-        k_state_roots<<<(unsigned)(gv > 0 ? gv : 1), 256, 0, st>>>(L, W, state, a16(L.labels));
-        k_state<<<(unsigned)(gv > 0 ? gv : 1), 256, 0, st>>>(L, state, a16(L.phi) && a16(L.labels) && a16(state));
+    const int64_t sxy = (int64_t)L.nx * L.ny;
+    // bits 0-3 of n as the low bits of four bytes
+    auto spread = [](uint32_t n) { return ((n & 15u) * 0x00204081u) & 0x01010101u; };
+    if (vec) {                                         // rows of whole 16-byte blocks
+        const int y = ti.y + tid % TY, z = ti.z + tid / TY;
+        if (y >= L.ny || z >= L.nz) return;
+        int8_t *out = state + (int64_t)z * sxy + (int64_t)y * L.nx + ti.x;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            uint32_t b[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) b[j] = spread(ones >> (16 * h + 4 * j)) | spread(ties >> (16 * h + 4 * j)) * 255u;
+            if (ti.x + 16 * h < L.nx)
+                __stcs(reinterpret_cast<int4 *>(out) + h, make_int4((int)b[0], (int)b[1], (int)b[2], (int)b[3]));
+        }
+        return;
     }
-    return cudaGetLastError();
+    row[tid] = make_uint2(ones, ties);
+    __syncthreads();
+    const int nrow = min(TZ, L.nz - ti.z) * TY;
+    for (int r = wid; r < nrow; r += NW) {
+        const int y = ti.y + r % TY, z = ti.z + r / TY;
+        if (y >= L.ny || ti.x + lane >= L.nx) continue;
+        const uint2 w = row[r];
+        state[(int64_t)z * sxy + (int64_t)y * L.nx + ti.x + lane] =
+            (int8_t)((w.x >> lane) & 1u ? 1 : ((w.y >> lane) & 1u ? -1 : 0));
+    }
 }
 
 // --------------------------------------------------------------------------------------
@@ -1479,7 +1527,7 @@ static int persistent_grid(K kernel, int threads, size_t smem, int64_t ntiles) {
 
 template <int TY, int TZ, int NL>
 static cudaError_t launch_all(const LatDev *lats, int n, const Plan &P, const Work &W, const PhiTmap *tms,
-                              cudaStream_t st, cudaEvent_t *ev, MergeSchedule ms) {
+                              cudaStream_t st, cudaEvent_t *ev, MergeSchedule ms, int8_t *state) {
     using SH = TileShape<TY, TZ>;
     LatBatch<NL> B;
     B.n = n;
@@ -1494,8 +1542,12 @@ static cudaError_t launch_all(const LatDev *lats, int n, const Plan &P, const Wo
         all_tma = all_tma && TB.tm[i].valid;
     }
     constexpr int CAP1 = LabelCfg<TY, TZ, true>::CAP, CAP1B = LabelCfg<TY, TZ, false>::CAP;
-    const size_t smem1 = sizeof(LabelSmem<TY, TZ, CAP1, LabelCfg<TY, TZ, true>::BL>);
-    const size_t smem1b = sizeof(LabelSmem<TY, TZ, CAP1B, LabelCfg<TY, TZ, false>::BL>);
+    constexpr int BL1 = LabelCfg<TY, TZ, true>::BL, BL1B = LabelCfg<TY, TZ, false>::BL;
+    constexpr bool IX = NL == 1;   // the index-field passes take one lattice
+    const bool index = IX && W.neg;
+    const size_t smem1 = sizeof(LabelSmem<TY, TZ, CAP1, BL1, false>);
+    const size_t smem1b = sizeof(LabelSmem<TY, TZ, CAP1B, BL1B, false>);
+    const size_t smem1x = sizeof(LabelSmem<TY, TZ, CAP1, BL1, IX>), smem1bx = sizeof(LabelSmem<TY, TZ, CAP1B, BL1B, IX>);
     const size_t smem4 = sizeof(FlatSmem<TY, TZ>);
     cudaError_t e;
     // Once per device a process uses: the shared-memory opt-ins (a device attribute of
@@ -1512,12 +1564,20 @@ static cudaError_t launch_all(const LatDev *lats, int n, const Plan &P, const Wo
         std::lock_guard<std::mutex> init_lock(init_mu);
         int *c = grid_cache[dev];
         if (!c[1]) {
-            e = cudaFuncSetAttribute(k_tile_label<TY, TZ, NL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            e = cudaFuncSetAttribute(k_tile_label<TY, TZ, NL, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)smem1);
             if (e != cudaSuccess) return e;
-            e = cudaFuncSetAttribute(k_tile_label<TY, TZ, NL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem1b);
+            e = cudaFuncSetAttribute(k_tile_label<TY, TZ, NL, false, false>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1b);
             if (e != cudaSuccess) return e;
+            if constexpr (IX) {
+                e = cudaFuncSetAttribute(k_tile_label<TY, TZ, 1, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem1x);
+                if (e != cudaSuccess) return e;
+                e = cudaFuncSetAttribute(k_tile_label<TY, TZ, 1, false, true>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1bx);
+                if (e != cudaSuccess) return e;
+            }
             e = cudaFuncSetAttribute(k_flatten<TY, TZ, NL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)smem4);
             if (e != cudaSuccess) return e;
@@ -1529,7 +1589,7 @@ static cudaError_t launch_all(const LatDev *lats, int n, const Plan &P, const Wo
             e = cudaFuncSetAttribute(k_occupancy_tma<TY, TZ, NL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)smem0);
             if (e != cudaSuccess) return e;
-            c[0] = persistent_grid(k_tile_label<TY, TZ, NL, false>, SH::NT, smem1b, INT32_MAX);
+            c[0] = persistent_grid(k_tile_label<TY, TZ, NL, false, IX>, SH::NT, smem1bx, INT32_MAX);
             c[2] = persistent_grid(k_occupancy_tma<TY, TZ, NL>, 256, smem0, INT32_MAX);
             c[1] = persistent_grid(k_flatten<TY, TZ, NL, false>, SH::NT, smem4, INT32_MAX);
         }
@@ -1549,10 +1609,15 @@ static cudaError_t launch_all(const LatDev *lats, int n, const Plan &P, const Wo
         launch_dep(k_occupancy<TY, TZ, NL>, (unsigned)((P.ntiles + 7) / 8), 256, 0, st, B, W, P.ntiles);
     }
     mark(1);
-    launch_dep(k_tile_label<TY, TZ, NL, true>, (unsigned)P.ntiles, SH::NT, smem1, st, B, W, P.ntiles);
-    // the tiles handed on (none for fields with at most MR_FAST / R runs a row on average)
-    launch_dep(k_tile_label<TY, TZ, NL, false>, (unsigned)(P.ntiles < grid1b ? P.ntiles : grid1b), SH::NT, smem1b, st,
-               B, W, P.ntiles);
+    // then the tiles handed on (none for fields with at most MR_FAST / R runs a row on average)
+    const unsigned g1b = (unsigned)(P.ntiles < grid1b ? P.ntiles : grid1b);
+    if (index) {
+        launch_dep(k_tile_label<TY, TZ, NL, true, IX>, (unsigned)P.ntiles, SH::NT, smem1x, st, B, W, P.ntiles);
+        launch_dep(k_tile_label<TY, TZ, NL, false, IX>, g1b, SH::NT, smem1bx, st, B, W, P.ntiles);
+    } else {
+        launch_dep(k_tile_label<TY, TZ, NL, true, false>, (unsigned)P.ntiles, SH::NT, smem1, st, B, W, P.ntiles);
+        launch_dep(k_tile_label<TY, TZ, NL, false, false>, g1b, SH::NT, smem1b, st, B, W, P.ntiles);
+    }
     mark(2);
     const unsigned gfm = (unsigned)((P.ntiles + FM_WARPS - 1) / FM_WARPS);
     if (ms.unions == 1) launch_dep(k_face_merge<TY, TZ, NL, 1>, gfm, 32 * FM_WARPS, 0, st, B, W, P.ntiles);
@@ -1564,6 +1629,16 @@ static cudaError_t launch_all(const LatDev *lats, int n, const Plan &P, const Wo
     if (ms.hot) launch_dep(k_piece_finalize<NL, true>, gpf, 32 * PF_WARPS, 0, st, B, W, P.ntiles, MB);
     else launch_dep(k_piece_finalize<NL, false>, gpf, 32 * PF_WARPS, 0, st, B, W, P.ntiles, MB);
     mark(4);
+    if constexpr (IX) {
+        if (state) {                               // index fields: the state is all that is wanted
+            mark(5);
+            mark(6);
+            const bool vec = (lats[0].nx & 15) == 0 && (reinterpret_cast<uintptr_t>(state) & 15) == 0;
+            launch_dep(k_state<TY, TZ>, (unsigned)P.ntiles, SH::NT, 0, st, lats[0], W, state, vec);
+            mark(7);
+            return launch_error != cudaSuccess ? launch_error : cudaGetLastError();
+        }
+    }
     const int64_t nb = (P.nrows + SCAN_CH) / SCAN_CH;   // covers index nrows (the total)
     const bool scanned = nb > SCAN_DIRECT;
     launch_dep(k_scan_reduce<NL>, (unsigned)nb, SCAN_NT, 0, st, B, (const uint8_t *)W.cnt, P.nrows, W.bsum);
@@ -1585,9 +1660,9 @@ static cudaError_t launch_all(const LatDev *lats, int n, const Plan &P, const Wo
 
 template <int TY, int TZ>
 static cudaError_t launch_shape(const LatDev *lats, int n, const Plan &P, const Work &W, const PhiTmap *tms,
-                                cudaStream_t st, cudaEvent_t *ev, MergeSchedule ms) {
-    if (n == 1) return launch_all<TY, TZ, 1>(lats, n, P, W, tms, st, ev, ms);
-    return launch_all<TY, TZ, MAX_LAT_PER_LAUNCH>(lats, n, P, W, tms, st, ev, ms);
+                                cudaStream_t st, cudaEvent_t *ev, MergeSchedule ms, int8_t *state) {
+    if (n == 1) return launch_all<TY, TZ, 1>(lats, n, P, W, tms, st, ev, ms, state);
+    return launch_all<TY, TZ, MAX_LAT_PER_LAUNCH>(lats, n, P, W, tms, st, ev, ms, nullptr);
 }
 
 template <int TY, int TZ>
@@ -1610,11 +1685,11 @@ bool tile_info(int ty, int tz, TileInfo &ti) {
 }
 
 cudaError_t launch_label(int ty, int tz, const LatDev *lats, int n, const Plan &P, const Work &W, const PhiTmap *tms,
-                         cudaStream_t st, cudaEvent_t *ev, MergeSchedule ms) {
-    if (ty == 8 && tz == 8) return launch_shape<8, 8>(lats, n, P, W, tms, st, ev, ms);
-    if (ty == 16 && tz == 8) return launch_shape<16, 8>(lats, n, P, W, tms, st, ev, ms);
-    if (ty == 16 && tz == 16) return launch_shape<16, 16>(lats, n, P, W, tms, st, ev, ms);
-    if (ty == 32 && tz == 8) return launch_shape<32, 8>(lats, n, P, W, tms, st, ev, ms);
+                         cudaStream_t st, cudaEvent_t *ev, MergeSchedule ms, int8_t *state) {
+    if (ty == 8 && tz == 8) return launch_shape<8, 8>(lats, n, P, W, tms, st, ev, ms, state);
+    if (ty == 16 && tz == 8) return launch_shape<16, 8>(lats, n, P, W, tms, st, ev, ms, state);
+    if (ty == 16 && tz == 16) return launch_shape<16, 16>(lats, n, P, W, tms, st, ev, ms, state);
+    if (ty == 32 && tz == 8) return launch_shape<32, 8>(lats, n, P, W, tms, st, ev, ms, state);
     return cudaErrorInvalidValue;
 }
 

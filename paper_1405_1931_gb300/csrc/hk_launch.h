@@ -36,12 +36,12 @@ constexpr int NUM_PASSES = 7;   // occupancy, tile_label, face_merge, piece_fina
 
 // Byte offsets of the workspace buffers of one launch (every offset 256-byte aligned).
 struct Layout {
-    size_t mask, codes, cnt, pre, face, tinfo, parent, key, psize, xcol, ovf, rootbits, segpre, votes, ncl, total;
+    size_t mask, codes, cnt, pre, face, tinfo, parent, key, psize, xcol, ovf, neg, pos, pvotes, tag, ncl, total;
 };
 
-// The workspace of one launch.  votes_cap > 0: also the root bits, the segment prefix
-// and the per-cluster votes of the interior/exterior identification (index fields).
-inline Layout make_layout(const TileInfo &ti, const Plan &P, int64_t votes_cap = 0) {
+// The workspace of one launch.  votes: also the sign words, the votes and the tags of the
+// interior/exterior identification (index fields).
+inline Layout make_layout(const TileInfo &ti, const Plan &P, bool votes = false) {
     Layout L{};
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -60,9 +60,10 @@ inline Layout make_layout(const TileInfo &ti, const Plan &P, int64_t votes_cap =
     L.psize = take((size_t)P.piece_cap * 4);
     L.xcol = take((size_t)P.ntiles * (ti.rows / 32) * 2 * 4);
     L.ovf = take((size_t)P.ntiles * 4);
-    L.rootbits = take(votes_cap > 0 ? (size_t)P.nseg * 4 : 0);
-    L.segpre = take(votes_cap > 0 ? (size_t)P.nseg * 4 : 0);
-    L.votes = take((size_t)votes_cap * 4);
+    L.neg = take(votes ? (size_t)P.ntiles * ti.rows * 4 : 0);
+    L.pos = take(votes ? (size_t)P.ntiles * ti.rows * 4 : 0);
+    L.pvotes = take(votes ? (size_t)P.piece_cap * 4 : 0);
+    L.tag = take(votes ? (size_t)P.ntiles * ti.maxruns / 4 : 0);
     L.ncl = take((size_t)MAX_LAT_PER_LAUNCH * 8);
     L.total = off;
     return L;
@@ -108,8 +109,11 @@ struct MergeSchedule {
 
 // ev: NUM_PASSES + 1 events recorded around the passes, or nullptr.  tms: the tensor
 // maps of each of the n lattices (valid == 0: the call takes the plain-load occupancy pass), or nullptr for none.
+// state != nullptr (one index field, W.neg set): the interior state of every site is
+// written instead of labels, sizes, histogram and count.
 cudaError_t launch_label(int ty, int tz, const LatDev *lats, int n, const Plan &P, const Work &W,
-                         const PhiTmap *tms, cudaStream_t st, cudaEvent_t *ev, MergeSchedule ms = MergeSchedule());
+                         const PhiTmap *tms, cudaStream_t st, cudaEvent_t *ev, MergeSchedule ms = MergeSchedule(),
+                         int8_t *state = nullptr);
 
 // The slab merge (hk_slab.cu): the face data of all R ranks and this rank's slab.
 struct SlabMerge {
@@ -139,10 +143,6 @@ cudaError_t launch_slab_faces(const int32_t *labels, int nx, int ny, int nzr, co
                               int32_t *list_lab, int64_t *list_size, int64_t *nf, cudaStream_t st);
 cudaError_t launch_slab_merge(const SlabMerge &M, cudaStream_t st);
 
-// Interior/exterior tags of a lattice labelled with occ_mode 1 (after launch_label on
-// the same stream; needs W.rootbits and W.votes).
-// state != nullptr: also the interior state of every site
-cudaError_t launch_interior(const LatDev &L, const Work &W, cudaStream_t st, int8_t *state = nullptr);
 // out[s] = the side index[s] names where the site is near a membrane (index >= -0.5 or
 // NaN), else prev[s]; out may be prev
 cudaError_t launch_interior_update(const int8_t *prev, const float *index, int64_t n, int8_t *out, cudaStream_t st);
