@@ -37,6 +37,7 @@ Work bind_work(char *base, const Layout &Ly, int32_t *status, int64_t piece_cap,
     W.ovf = reinterpret_cast<int32_t *>(base + Ly.ovf);
     W.neg = reinterpret_cast<uint32_t *>(base + Ly.neg);
     W.pos = reinterpret_cast<uint32_t *>(base + Ly.pos);
+    W.near_tile = reinterpret_cast<uint32_t *>(base + Ly.near_tile);
     W.pvotes = reinterpret_cast<int32_t *>(base + Ly.pvotes);
     W.tag = reinterpret_cast<uint32_t *>(base + Ly.tag);
     W.novf = status + 1;
@@ -390,7 +391,7 @@ int run_lattices(hk_ctx *ctx, const hk_lattice *lats, int n, cudaStream_t st, bo
         char *base = static_cast<char *>(ctx->ws);
         Work W = hk::bind_work(base, Ly, ctx->dstatus, P.piece_cap, ctx->loop_cap);
         if (!inside && !state) {
-            W.neg = W.pos = W.tag = nullptr;
+            W.neg = W.pos = W.near_tile = W.tag = nullptr;
             W.pvotes = nullptr;
         }
         W.site_off = site_off;   // slab calls: one lattice

@@ -26,6 +26,8 @@ constexpr int TX = 32;
 constexpr uint16_t CODE_BOUNDARY = 0x8000;
 constexpr uint16_t CODE_ROOT = 0x4000;
 constexpr uint16_t CODE_LOW = 0x3fff;
+// Tile record flag: all runs of the tile are boundary piece 0.
+constexpr int TILE_ONE_PIECE = 1 << 30;
 
 // One lattice of a launch.  Every pass works on the concatenated tiles of all
 // lattices; tile0/seg0/row0 locate this lattice's slice of the global tile,
@@ -65,7 +67,8 @@ struct Work {
     uint32_t *bsum;     // [nblocks] scan block sums (in face's space, which is free by then)
     uint16_t *face;     // [ntiles * face_stride] per-face lists of boundary-piece numbers
     int4 *tinfo;        // [ntiles] each tile's first site (x, y, z) and its counts: boundary pieces
-                        // (bits 0-10), runs (bits 11-23), lattice of the launch (bits 24-29)
+                        // (bits 0-10), runs (bits 11-23), lattice of the launch (bits 24-29),
+                        // TILE_ONE_PIECE (index fields)
     int32_t *parent;    // [piece_cap] union-find parent over boundary pieces; tile t owns
                         // the slice [t * MAX_BOUNDARY, t * MAX_BOUNDARY + piece count)
     int32_t *key;       // [piece_cap] lattice-local site index of the piece's first site;
@@ -81,6 +84,7 @@ struct Work {
     // pieces per run the tag that the votes give (two words per 32 runs: bit set where
     // interior, bit set where undetermined)
     uint32_t *neg, *pos;
+    uint32_t *near_tile;   // [ntiles] whether the tile has near sites with a sign
     int32_t *pvotes;    // [piece_cap]
     uint32_t *tag;      // [ntiles * MAXRUNS / 16]
     int32_t *ovf;       // [ntiles] tiles with more runs than the fast tile pass holds

@@ -58,6 +58,7 @@ __global__ void __launch_bounds__(256, 4) k_occupancy(const __grid_constant__ La
     const bool vec = g.lastX == TX - 1 && (L.nx & 3) == 0 && (reinterpret_cast<uintptr_t>(L.phi) & 15) == 0;
     const int x4 = (lane & 7) * 4;
     const float *base4 = L.phi + (int64_t)g.z0 * sxy + (int64_t)g.y0 * L.nx + g.x0 + x4;
+    uint32_t any_near = 0;
     for (int r0 = 0; r0 < R; r0 += 32) {        // lane j keeps the words of row r0 + j
         uint32_t mine = 0, neg = 0, pos = 0;
         if (vec) {
@@ -119,6 +120,7 @@ __global__ void __launch_bounds__(256, 4) k_occupancy(const __grid_constant__ La
         if (W.neg) {
             W.neg[t * R + r0 + lane] = neg;
             W.pos[t * R + r0 + lane] = pos;
+            any_near |= neg | pos;
         }
         // first and last column of the tile, one bit per row (faces along x)
         const uint32_t c0 = __ballot_sync(0xffffffffu, mine & 1u);
@@ -127,6 +129,10 @@ __global__ void __launch_bounds__(256, 4) k_occupancy(const __grid_constant__ La
             W.xcol[(t * 2) * (R / 32) + (r0 >> 5)] = c0;
             W.xcol[(t * 2 + 1) * (R / 32) + (r0 >> 5)] = cl;
         }
+    }
+    if (W.neg) {
+        any_near = __reduce_or_sync(0xffffffffu, any_near);
+        if (lane == 0) W.near_tile[t] = any_near != 0u;
     }
 }
 
@@ -140,7 +146,9 @@ struct OccSmem {
     uint64_t bar[2];
 };
 
-template <int TY, int TZ, int NL>
+// INDEX: also the signs of the near sites (its own instance: three votes a row, and a
+// batch of plain fields took 381 against 333 us with the choice made at run time).
+template <int TY, int TZ, int NL, bool INDEX>
 __global__ void __launch_bounds__(256) k_occupancy_tma(const __grid_constant__ TmapBatch<NL> TB,
                                                        const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
     grid_dep_wait();
@@ -183,25 +191,34 @@ __global__ void __launch_bounds__(256) k_occupancy_tma(const __grid_constant__ T
         const LatDev &L = B.lat[(NL == 1) ? 0 : find_lattice(B.lat, B.n, t)];
         const int lastX = tile_geo<TY, TZ>(L, t).lastX;
         // warp w converts rows [32 w', 32 w' + 32) in turns; lane j keeps row 32 w' + j
+        [[maybe_unused]] uint32_t any_near = 0;
         for (int r0 = wid * 32; r0 < R; r0 += 32 * (256 / 32)) {
             uint32_t mine = 0;
-#pragma unroll 8
-            for (int j = 0; j < 32; ++j) {
-                const uint32_t w = __ballot_sync(0xffffffffu, occupied(S.buf[s][(r0 + j) * 32 + lane], L.occ_mode));
-                if (lane == j) mine = w;
-            }
-            W.mask[t * R + r0 + lane] = mine;
-            if (W.neg) {                               // uniform: signs of the near sites
+            if constexpr (INDEX) {
                 uint32_t neg = 0, pos = 0;
 #pragma unroll 8
                 for (int j = 0; j < 32; ++j) {
-                    const uint32_t n = near_bits(S.buf[s][(r0 + j) * 32 + lane], 0);
-                    const uint32_t wn = __ballot_sync(0xffffffffu, n & 1u), wp = __ballot_sync(0xffffffffu, n >> 16);
-                    if (lane == j) { neg = wn; pos = wp; }
+                    const float v = S.buf[s][(r0 + j) * 32 + lane];
+                    const uint32_t w = __ballot_sync(0xffffffffu, occupied(v, 1));
+                    const uint32_t wn = __ballot_sync(0xffffffffu, v < 0.0f), wp = __ballot_sync(0xffffffffu, v > 0.0f);
+                    if (lane == j) {
+                        mine = w;
+                        neg = wn;
+                        pos = wp;
+                    }
                 }
+                neg &= ~mine;                          // near and negative; a positive site is never far
                 W.neg[t * R + r0 + lane] = neg;
                 W.pos[t * R + r0 + lane] = pos;
+                any_near |= neg | pos;
+            } else {
+#pragma unroll 8
+                for (int j = 0; j < 32; ++j) {
+                    const uint32_t w = __ballot_sync(0xffffffffu, occupied(S.buf[s][(r0 + j) * 32 + lane], L.occ_mode));
+                    if (lane == j) mine = w;
+                }
             }
+            W.mask[t * R + r0 + lane] = mine;
             const uint32_t c0 = __ballot_sync(0xffffffffu, mine & 1u);
             const uint32_t cl = __ballot_sync(0xffffffffu, (mine >> lastX) & 1u);
             if (lane == 0) {
@@ -209,7 +226,13 @@ __global__ void __launch_bounds__(256) k_occupancy_tma(const __grid_constant__ T
                 W.xcol[(t * 2 + 1) * (R / 32) + (r0 >> 5)] = cl;
             }
         }
-        __syncthreads();                       // every warp is done with buffer s
+        // every warp is done with buffer s
+        if constexpr (INDEX) {
+            const bool near_tile = __syncthreads_or(any_near != 0u);
+            if (tid == 0) W.near_tile[t] = near_tile;
+        } else {
+            __syncthreads();
+        }
         if (tid == 0 && t + 2 * step < ntiles) issue(t + 2 * step, s);
     }
 }
@@ -243,6 +266,7 @@ struct LabelSmem {
     static_assert(SH::R <= 256 && CAP <= 4096, "desc holds an 8-bit row and run ids fit in 16 bits");
     uint32_t rowcnt[SH::R / 4];            // interior roots of each row, a byte each
     int nbnd;                              // boundary roots of the tile
+    int nint;                              // interior roots (index fields)
     int warp_tmp[32];
     uint32_t neg[INDEX ? SH::R : 1], pos[INDEX ? SH::R : 1];   // signs of the near sites of each row
     int votes[INDEX ? CAP : 1];            // per root: the votes of its piece's sites
@@ -253,13 +277,18 @@ constexpr int DESC_TOUCH = 1 << 13;  // desc flag: the run has a site connected 
 
 // Resident CTAs per SM of the fast tile pass (its shared memory and 32 registers a
 // thread allow 2048 threads) and of the pass over the tiles it hands on.
-template <int TY, int TZ, bool FAST>
+// Index fields whose votes are wanted hold fewer runs a row (membranes and bulk fluid), for
+// room for their votes: 4 on average.
+template <int TY, int TZ, bool FAST, bool INDEX = false>
 struct LabelCfg {
-    static constexpr int CAP = FAST ? TileShape<TY, TZ>::MR_FAST : TileShape<TY, TZ>::MAXRUNS;
+    static constexpr int CAP = !FAST ? TileShape<TY, TZ>::MAXRUNS
+                             : INDEX ? 4 * TileShape<TY, TZ>::R : TileShape<TY, TZ>::MR_FAST;
     // boundary pieces the fast pass lists (more go to the second pass, which has room for all)
     static constexpr int BL = FAST && TileShape<TY, TZ>::MAX_BOUNDARY > 512 ? 512 : TileShape<TY, TZ>::MAX_BOUNDARY;
-    static constexpr int BLOCKS = FAST ? (2048 / (TY * TZ) < 32 ? 2048 / (TY * TZ) : 32)
-                                       : (1280 / (TY * TZ) < 32 ? 1280 / (TY * TZ) : 32);
+    // resident threads of an SM; index fields wait more than they issue (729 capsules at
+    // 1024^3: 1.34 ms at 1280, 1.19 at 1536, 1.11 at 1792 and 2048)
+    static constexpr int THREADS = !FAST ? 1280 : INDEX ? 1792 : 2048;
+    static constexpr int BLOCKS = THREADS / (TY * TZ) < 32 ? THREADS / (TY * TZ) : 32;
 };
 
 // FAST: tiles t = blockIdx.x, blockIdx.x + gridDim.x, ... below ntiles; a tile with
@@ -267,12 +296,12 @@ struct LabelCfg {
 // !FAST: the tiles listed in W.ovf, with room for every tile.
 // INDEX: an index field whose clusters' votes are wanted (Sec. 6, step 5; one lattice).
 template <int TY, int TZ, int NL, bool FAST, bool INDEX>
-__global__ void __launch_bounds__(TY * TZ, (LabelCfg<TY, TZ, FAST && !INDEX>::BLOCKS))
+__global__ void __launch_bounds__(TY * TZ, (LabelCfg<TY, TZ, FAST, INDEX>::BLOCKS))
 k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
     grid_dep_wait();
     using SH = TileShape<TY, TZ>;
-    constexpr int R = SH::R, NT = SH::NT, MR = SH::MAXRUNS, CAP = LabelCfg<TY, TZ, FAST>::CAP;
-    constexpr int BL = LabelCfg<TY, TZ, FAST>::BL;
+    constexpr int R = SH::R, NT = SH::NT, MR = SH::MAXRUNS, CAP = LabelCfg<TY, TZ, FAST, INDEX>::CAP;
+    constexpr int BL = LabelCfg<TY, TZ, FAST, INDEX>::BL;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     LabelSmem<TY, TZ, CAP, BL, INDEX> &S = *reinterpret_cast<LabelSmem<TY, TZ, CAP, BL, INDEX> *>(smem_raw);
     const int tid = threadIdx.x;
@@ -287,9 +316,22 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
         const int r = tid, ly = r % TY, lz = r / TY;
         const uint32_t m = W.mask[t * R + r];
         S.m[r] = m;
+        bool near_here = false;                   // CTA-uniform: the tile or one across a face has near sites
         if (INDEX) {
-            S.neg[r] = W.neg[t * R + r];
-            S.pos[r] = W.pos[t * R + r];
+            const int64_t plane = (int64_t)L.nbx * L.nby;
+            const int64_t nb[7] = {t, g.bx > 0 ? t - 1 : t + (L.nbx - 1), g.bx < L.nbx - 1 ? t + 1 : t - (L.nbx - 1),
+                                   g.by > 0 ? t - L.nbx : t + (int64_t)(L.nby - 1) * L.nbx,
+                                   g.by < L.nby - 1 ? t + L.nbx : t - (int64_t)(L.nby - 1) * L.nbx,
+                                   g.bz > 0 ? t - plane : t + (int64_t)(L.nbz - 1) * plane,
+                                   g.bz < L.nbz - 1 ? t + plane : t - (int64_t)(L.nbz - 1) * plane};
+            uint32_t any = 0;
+#pragma unroll
+            for (int k = 0; k < 7; ++k) any |= W.near_tile[nb[k]];
+            near_here = any != 0u;
+            if (near_here) {
+                S.neg[r] = W.neg[t * R + r];
+                S.pos[r] = W.pos[t * R + r];
+            }
         }
         const uint32_t rs = run_starts(m);
         {
@@ -447,7 +489,7 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
 
         // Sizes accumulate in aux, which held the pair lists until the unions above.
         if (tid < R / 4) S.rowcnt[tid] = 0u;
-        if (tid == 0) S.nbnd = 0;
+        if (tid == 0) S.nbnd = S.nint = 0;
         for (int i = 4 * tid; i < total; i += 4 * NT)
             *reinterpret_cast<int4 *>(&S.aux[i]) = make_int4(0, 0, 0, 0);
         if (INDEX)
@@ -474,7 +516,7 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
         // of its sites are words like its own (a row of the tile, of the tile across a face
         // or across a periodic edge, or its own word moved by one along x), so a run's votes
         // are counts of bits; rows away from every membrane have none.
-        if (INDEX && m) {
+        if (INDEX && near_here && m) {
             const int64_t plane = (int64_t)L.nbx * L.nby;
             auto row_of = [&](const uint32_t *sw, const uint32_t *gw, int axis, bool hi) -> uint32_t {
                 const int c = axis == 1 ? ly : lz, last = axis == 1 ? g.lastY : g.lastZ, step = axis == 1 ? 1 : TY;
@@ -538,6 +580,7 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
                 if (root && !bnd) {
                     const int row = (S.desc[i] >> 5) & 0xff;
                     atomicAdd(&S.rowcnt[row >> 2], 1u << (8 * (row & 3)));   // a byte a row: at most 16
+                    if (INDEX) S.nint = 1;
                 }
             }
         }
@@ -560,7 +603,7 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
         }
         if (tid == 0)
             W.tinfo[t] = make_int4(g.x0, g.y0, g.z0,
-                                   nb_ | (total << 11) | (lat << 24));
+                                   nb_ | (total << 11) | (lat << 24) | (INDEX && nb_ == 1 && !S.nint ? TILE_ONE_PIECE : 0));
         __syncthreads();
 
         // interior roots per row segment
@@ -582,7 +625,7 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
             C[i] = c;
         }
 
-        if (INDEX) {                              // the tag of each run's piece, as if it were interior
+        if (INDEX && S.nint) {                    // the tag of each run's piece, as if it were interior
             const int lane = tid & 31;
             uint32_t *T = W.tag + t * (MR / 16);
             for (int i0 = tid - lane; i0 < total; i0 += NT) {
@@ -1317,7 +1360,9 @@ k_flatten(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles, uint32
 // site the side its value names (step 2: -d inside, +d outside), 1 for I < 0 and 0
 // otherwise.  Like flatten it decodes the runs of each tile, but it needs neither ranks
 // nor labels: it reads the words and codes and writes a byte a site.  One tile per CTA,
-// one row per thread.
+// one row per thread; a tile of one piece, as most are, needs no codes.  Bound by the
+// latency of its few loads: 729 capsules at 1024^3 take 0.30 ms, a fifth of the copy
+// rate for its 1.3 GB (0.51 with codes read in every tile and half sectors stored).
 // --------------------------------------------------------------------------------------
 template <int TY, int TZ>
 __global__ void __launch_bounds__(TY * TZ) k_state(const LatDev L, Work W, int8_t *state, bool vec) {
@@ -1332,52 +1377,61 @@ __global__ void __launch_bounds__(TY * TZ) k_state(const LatDev L, Work W, int8_
     const int4 ti = W.tinfo[t];
     const int nb = ti.w & 0x7ff;
     const uint32_t m = W.mask[t * R + tid], near_in = W.neg[t * R + tid];
+    const int root0 = W.parent[t * MB];                // of piece 0, if there is one
     const uint32_t rs = run_starts(m);
-    int inc = __popc(rs);
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const int u = __shfl_up_sync(0xffffffffu, inc, d);
-        if (lane >= d) inc += u;
-    }
-    if (lane == 31) warp_tmp[wid] = inc;
-    for (int k = tid; k < nb; k += NT) {
-        const int v = W.pvotes[W.parent[t * MB + k]];  // piece_finalize left every piece at its root
-        ptag[k] = (int8_t)(v < 0 ? 1 : (v > 0 ? 0 : -1));
-    }
-    __syncthreads();
-    int id = inc - __popc(rs);
-#pragma unroll
-    for (int w = 0; w < NW; ++w)
-        if (w < wid) id += warp_tmp[w];
     uint32_t ones = near_in, ties = 0;
-    for (uint32_t w = rs; w; ++id) {
-        const uint32_t low = w & (0u - w), run = fill_up(m, low);
-        w ^= low;
-        const int c = __ldg(W.codes + t * MR + id);
-        int tag;
-        if (c & CODE_BOUNDARY) {
-            tag = ptag[c & CODE_LOW];
-        } else {
-            const uint32_t *T = W.tag + t * (MR / 16) + 2 * (id >> 5);
-            tag = (__ldg(T) >> (id & 31)) & 1u ? 1 : ((__ldg(T + 1) >> (id & 31)) & 1u ? -1 : 0);
+    if (ti.w & TILE_ONE_PIECE) {                       // uniform: the tile's far sites are one piece
+        const int v = W.pvotes[root0];
+        if (v < 0) ones |= m;
+        if (v == 0) ties = m;
+    } else {
+        int inc = __popc(rs);
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, inc, d);
+            if (lane >= d) inc += u;
         }
-        if (tag > 0) ones |= run;
-        if (tag < 0) ties |= run;
+        if (lane == 31) warp_tmp[wid] = inc;
+        for (int k = tid; k < nb; k += NT) {
+            const int v = W.pvotes[W.parent[t * MB + k]];  // piece_finalize left every piece at its root
+            ptag[k] = (int8_t)(v < 0 ? 1 : (v > 0 ? 0 : -1));
+        }
+        __syncthreads();
+        int id = inc - __popc(rs);
+#pragma unroll
+        for (int w = 0; w < NW; ++w)
+            if (w < wid) id += warp_tmp[w];
+        for (uint32_t w = rs; w; ++id) {
+            const uint32_t low = w & (0u - w), run = fill_up(m, low);
+            w ^= low;
+            const int c = __ldg(W.codes + t * MR + id);
+            int tag;
+            if (c & CODE_BOUNDARY) {
+                tag = ptag[c & CODE_LOW];
+            } else {
+                const uint32_t *T = W.tag + t * (MR / 16) + 2 * (id >> 5);
+                tag = (__ldg(T) >> (id & 31)) & 1u ? 1 : ((__ldg(T + 1) >> (id & 31)) & 1u ? -1 : 0);
+            }
+            if (tag > 0) ones |= run;
+            if (tag < 0) ties |= run;
+        }
     }
     const int64_t sxy = (int64_t)L.nx * L.ny;
     // bits 0-3 of n as the low bits of four bytes
     auto spread = [](uint32_t n) { return ((n & 15u) * 0x00204081u) & 0x01010101u; };
-    if (vec) {                                         // rows of whole 16-byte blocks
-        const int y = ti.y + tid % TY, z = ti.z + tid / TY;
-        if (y >= L.ny || z >= L.nz) return;
-        int8_t *out = state + (int64_t)z * sxy + (int64_t)y * L.nx + ti.x;
+    if (vec) {      // rows of whole 16-byte blocks: two lanes a row, so that a store fills sectors
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
+            const int r = wid * 32 + h * 16 + (lane >> 1), x = 16 * (lane & 1);
+            const uint32_t o = __shfl_sync(0xffffffffu, ones, h * 16 + (lane >> 1)) >> x;
+            const uint32_t e = __shfl_sync(0xffffffffu, ties, h * 16 + (lane >> 1)) >> x;
             uint32_t b[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = spread(ones >> (16 * h + 4 * j)) | spread(ties >> (16 * h + 4 * j)) * 255u;
-            if (ti.x + 16 * h < L.nx)
-                __stcs(reinterpret_cast<int4 *>(out) + h, make_int4((int)b[0], (int)b[1], (int)b[2], (int)b[3]));
+            for (int j = 0; j < 4; ++j) b[j] = spread(o >> (4 * j)) | spread(e >> (4 * j)) * 255u;
+            const int y = ti.y + r % TY, z = ti.z + r / TY;
+            if (y < L.ny && z < L.nz && ti.x + x < L.nx)
+                __stcs(reinterpret_cast<int4 *>(state + (int64_t)z * sxy + (int64_t)y * L.nx + ti.x + x),
+                       make_int4((int)b[0], (int)b[1], (int)b[2], (int)b[3]));
         }
         return;
     }
@@ -1547,7 +1601,7 @@ static cudaError_t launch_all(const LatDev *lats, int n, const Plan &P, const Wo
     const bool index = IX && W.neg;
     const size_t smem1 = sizeof(LabelSmem<TY, TZ, CAP1, BL1, false>);
     const size_t smem1b = sizeof(LabelSmem<TY, TZ, CAP1B, BL1B, false>);
-    const size_t smem1x = sizeof(LabelSmem<TY, TZ, CAP1, BL1, IX>), smem1bx = sizeof(LabelSmem<TY, TZ, CAP1B, BL1B, IX>);
+    const size_t smem1x = sizeof(LabelSmem<TY, TZ, LabelCfg<TY, TZ, true, IX>::CAP, BL1, IX>), smem1bx = sizeof(LabelSmem<TY, TZ, CAP1B, BL1B, IX>);
     const size_t smem4 = sizeof(FlatSmem<TY, TZ>);
     cudaError_t e;
     // Once per device a process uses: the shared-memory opt-ins (a device attribute of
@@ -1586,11 +1640,16 @@ static cudaError_t launch_all(const LatDev *lats, int n, const Plan &P, const Wo
                                          (int)smem4);
                 if (e != cudaSuccess) return e;
             }
-            e = cudaFuncSetAttribute(k_occupancy_tma<TY, TZ, NL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            e = cudaFuncSetAttribute(k_occupancy_tma<TY, TZ, NL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)smem0);
             if (e != cudaSuccess) return e;
+            if constexpr (IX) {
+                e = cudaFuncSetAttribute(k_occupancy_tma<TY, TZ, NL, IX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem0);
+                if (e != cudaSuccess) return e;
+            }
             c[0] = persistent_grid(k_tile_label<TY, TZ, NL, false, IX>, SH::NT, smem1bx, INT32_MAX);
-            c[2] = persistent_grid(k_occupancy_tma<TY, TZ, NL>, 256, smem0, INT32_MAX);
+            c[2] = persistent_grid(k_occupancy_tma<TY, TZ, NL, IX>, 256, smem0, INT32_MAX);
             c[1] = persistent_grid(k_flatten<TY, TZ, NL, false>, SH::NT, smem4, INT32_MAX);
         }
         grid1b = c[0];
@@ -1604,7 +1663,8 @@ static cudaError_t launch_all(const LatDev *lats, int n, const Plan &P, const Wo
     mark(0);
     if (all_tma) {
         const unsigned g0 = (unsigned)(P.ntiles < grid0 ? P.ntiles : grid0);
-        launch_dep(k_occupancy_tma<TY, TZ, NL>, g0, 256, smem0, st, TB, B, W, P.ntiles);
+        if (index) launch_dep(k_occupancy_tma<TY, TZ, NL, IX>, g0, 256, smem0, st, TB, B, W, P.ntiles);
+        else launch_dep(k_occupancy_tma<TY, TZ, NL, false>, g0, 256, smem0, st, TB, B, W, P.ntiles);
     } else {
         launch_dep(k_occupancy<TY, TZ, NL>, (unsigned)((P.ntiles + 7) / 8), 256, 0, st, B, W, P.ntiles);
     }

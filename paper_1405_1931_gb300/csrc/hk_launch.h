@@ -36,7 +36,7 @@ constexpr int NUM_PASSES = 7;   // occupancy, tile_label, face_merge, piece_fina
 
 // Byte offsets of the workspace buffers of one launch (every offset 256-byte aligned).
 struct Layout {
-    size_t mask, codes, cnt, pre, face, tinfo, parent, key, psize, xcol, ovf, neg, pos, pvotes, tag, ncl, total;
+    size_t mask, codes, cnt, pre, face, tinfo, parent, key, psize, xcol, ovf, neg, pos, near_tile, pvotes, tag, ncl, total;
 };
 
 // The workspace of one launch.  votes: also the sign words, the votes and the tags of the
@@ -62,6 +62,7 @@ inline Layout make_layout(const TileInfo &ti, const Plan &P, bool votes = false)
     L.ovf = take((size_t)P.ntiles * 4);
     L.neg = take(votes ? (size_t)P.ntiles * ti.rows * 4 : 0);
     L.pos = take(votes ? (size_t)P.ntiles * ti.rows * 4 : 0);
+    L.near_tile = take(votes ? (size_t)P.ntiles * 4 : 0);
     L.pvotes = take(votes ? (size_t)P.piece_cap * 4 : 0);
     L.tag = take(votes ? (size_t)P.ntiles * ti.maxruns / 4 : 0);
     L.ncl = take((size_t)MAX_LAT_PER_LAUNCH * 8);

@@ -94,7 +94,7 @@ extern "C" int hk_label_noalloc(const float *phi, int nx, int ny, int nz, const 
     // read (here on the capacity path, or by hk_noalloc_sync_status), so a give-up is
     // reported even when several calls run before the check.
     hk::Work W = hk::bind_work(base + HEADER_BYTES, Ly, reinterpret_cast<int32_t *>(base), P.piece_cap, 0);
-    W.neg = W.pos = W.tag = nullptr;   // no interior/exterior identification here
+    W.neg = W.pos = W.near_tile = W.tag = nullptr;   // no interior/exterior identification here
     W.pvotes = nullptr;
 
     hk::LatDev d;
