@@ -1486,6 +1486,39 @@ __global__ void __launch_bounds__(256) k_interior_update(const int8_t *prev, con
     }
 }
 
+// Dense form in place: a far site's state stays where it is, so only the groups of four
+// sites that hold a near one are read and written (one in fifty for 729 capsules at
+// 1024^3), and the pass is the read of the index field: 0.97 ms with every state moved,
+// 0.66 ms so.  Four 16-byte index loads in flight a thread.  vec: index 16-byte and state
+// 4-byte aligned.
+__global__ void __launch_bounds__(256) k_interior_update_in_place(int8_t *state, const float *index, int64_t n,
+                                                                   bool vec) {
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+    int64_t done = 0;
+    if (vec) {
+        constexpr int U = 4;
+        const int64_t nv = n / 4;
+        for (int64_t i0 = t0; i0 < nv; i0 += U * stride) {
+            float4 v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                v[u] = i0 + u * stride < nv ? __ldcs(reinterpret_cast<const float4 *>(index) + i0 + u * stride)
+                                            : make_float4(-1.f, -1.f, -1.f, -1.f);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (v[u].x < -0.5f && v[u].y < -0.5f && v[u].z < -0.5f && v[u].w < -0.5f) continue;
+                uint32_t *p = reinterpret_cast<uint32_t *>(state) + i0 + u * stride;
+                *p = update_byte(update_byte(update_byte(update_byte(*p, 0, v[u].x), 1, v[u].y), 2, v[u].z), 3, v[u].w);
+            }
+        }
+        done = nv * 4;
+    }
+    for (int64_t s = done + t0; s < n; s += stride) {
+        const float v = index[s];
+        if (!(v < -0.5f)) state[s] = (int8_t)(v < 0.0f ? 1 : 0);
+    }
+}
+
 // Sparse form: the caller lists the near sites with their values.
 __global__ void __launch_bounds__(256) k_interior_update_sites(int8_t *state, int64_t n, const int32_t *sites,
                                                                 const float *values, int64_t m) {
@@ -1508,6 +1541,11 @@ static unsigned stream_grid(int64_t units) {
 
 cudaError_t launch_interior_update(const int8_t *prev, const float *index, int64_t n, int8_t *out, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
+    if (prev == out) {
+        const bool vec = (reinterpret_cast<uintptr_t>(index) & 15) == 0 && (reinterpret_cast<uintptr_t>(out) & 3) == 0;
+        k_interior_update_in_place<<<stream_grid(vec ? n / 16 + 1 : n), 256, 0, st>>>(out, index, n, vec);
+        return cudaGetLastError();
+    }
     const bool vec = ((reinterpret_cast<uintptr_t>(prev) | reinterpret_cast<uintptr_t>(index) |
                        reinterpret_cast<uintptr_t>(out)) & 15) == 0;
     k_interior_update<<<stream_grid(vec ? n / 16 + 1 : n), 256, 0, st>>>(prev, index, n, out, vec);
