@@ -240,13 +240,11 @@ __global__ void __launch_bounds__(256) k_occupancy_tma(const __grid_constant__ T
 // --------------------------------------------------------------------------------------
 // K1: tile labelling from the occupancy words (one tile per CTA)
 //
-// Bound by instruction issue (90 % of its rate): 2.2 warp instructions a site at p_c.
-// With most pairs linked or left out instead of united, and with boundary roots listed
-// by a counter instead of two passes and a scan over all runs: 2.11 against 2.38 ms at
-// 1024^3, p_c, 0.83 against 1.06 ms on blocks of 16^3, 0.130 against 0.148 ms on a 512^3
-// bijel.  Where it goes at p_c (cumulative cuts): loads and geometry 0.22 ms, run ids and
-// nodes 0.16, pair words and their scan 0.06, links and lists 0.17, unions 0.30,
-// compression and sizes 0.39, boundary pieces 0.41, row counts 0.04, codes 0.18, faces 0.18.
+// Bound by instruction issue (90 % of its rate): 2 warp instructions a site at p_c.  With
+// most pairs linked or left out instead of united, and with boundary pieces listed by the
+// run that first touches a face instead of in passes over all runs: 1.93 against 2.38 ms
+// at 1024^3, p_c, 0.81 against 1.06 ms on blocks of 16^3, 0.127 against 0.148 ms on a
+// 512^3 bijel.
 // --------------------------------------------------------------------------------------
 template <int TY, int TZ, int CAP, int BL, bool INDEX>
 struct LabelSmem {
@@ -264,9 +262,9 @@ struct LabelSmem {
     uint32_t xo0[SH::R / 32], xol[SH::R / 32];     // this tile's first and last column
     static_assert(TZ <= 16 && TY <= 32 && SH::R / 32 <= 16 && SH::NT >= 64, "face loads use threads 0..63");
     static_assert(SH::R <= 256 && CAP <= 4096, "desc holds an 8-bit row and run ids fit in 16 bits");
-    uint32_t rowcnt[SH::R / 4];            // interior roots of each row, a byte each
+    uint32_t rowcnt[SH::R / 4];            // roots, then interior roots of each row, a byte each
     int nbnd;                              // boundary roots of the tile
-    int nint;                              // interior roots (index fields)
+    int nroot;                             // roots (index fields)
     int warp_tmp[32];
     uint32_t neg[INDEX ? SH::R : 1], pos[INDEX ? SH::R : 1];   // signs of the near sites of each row
     int votes[INDEX ? CAP : 1];            // per root: the votes of its piece's sites
@@ -489,7 +487,7 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
 
         // Sizes accumulate in aux, which held the pair lists until the unions above.
         if (tid < R / 4) S.rowcnt[tid] = 0u;
-        if (tid == 0) S.nbnd = S.nint = 0;
+        if (tid == 0) S.nbnd = S.nroot = 0;
         for (int i = 4 * tid; i < total; i += 4 * NT)
             *reinterpret_cast<int4 *>(&S.aux[i]) = make_int4(0, 0, 0, 0);
         if (INDEX)
@@ -500,14 +498,27 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
         // first run), and the run's length -- plus AUX_FACE if it touches a face -- is
         // added to its root.  The finds are read-only, so storing final roots while
         // others still search is safe.  A piece is a boundary piece iff its sum reaches
-        // AUX_FACE (sizes stay below it).
+        // AUX_FACE (sizes stay below it): the run that brings its root there lists it and
+        // gives the piece its number (in any order: a number only names the piece).  The
+        // roots of each row are counted, a byte a row (at most 16).
         for (int i = tid; i < total; i += NT) {
             int root = S.par[i];
             for (int up = S.par[root]; up != root; up = S.par[root]) root = S.par[up];   // two levels a step
             S.par[i] = root;
-            const int d = S.desc[i];
-            const int len = run_len(S.m[(d >> 5) & 0xff], d & 31);
-            atomicAdd(&S.aux[root], len + ((d & DESC_TOUCH) ? AUX_FACE : 0));
+            const int d = S.desc[i], row = (d >> 5) & 0xff;
+            const int len = run_len(S.m[row], d & 31);
+            if (d & DESC_TOUCH) {
+                if (atomicAdd(&S.aux[root], len + AUX_FACE) < AUX_FACE) {
+                    const int k = atomicAdd(&S.nbnd, 1);
+                    if (k < BL) S.blist[k] = (uint16_t)root;
+                }
+            } else {
+                atomicAdd(&S.aux[root], len);
+            }
+            if (root == i) {
+                atomicAdd(&S.rowcnt[row >> 2], 1u << (8 * (row & 3)));
+                if (INDEX) atomicAdd(&S.nroot, 1);
+            }
         }
         __syncthreads();
 
@@ -561,30 +572,8 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
         }
         if (INDEX) __syncthreads();
 
-        // Number the boundary roots (in any order: the number only names the piece) and list
-        // them, so that only they do the record writes; interior roots are counted per row.
+        // the boundary pieces' records
         const int base = (int)(t * SH::MAX_BOUNDARY);   // fixed slice of the piece table
-        {
-            const int lane = tid & 31;
-            for (int i0 = tid - lane; i0 < total; i0 += NT) {
-                const int i = i0 + lane;
-                const bool root = i < total && S.par[i] == i;
-                const bool bnd = root && S.aux[i] >= AUX_FACE;
-                const uint32_t bal = __ballot_sync(0xffffffffu, bnd);
-                if (bal) {
-                    int k0 = 0;
-                    if (lane == 0) k0 = atomicAdd(&S.nbnd, __popc(bal));
-                    const int k = __shfl_sync(0xffffffffu, k0, 0) + __popc(bal & ((1u << lane) - 1u));
-                    if (bnd && k < BL) S.blist[k] = (uint16_t)i;
-                }
-                if (root && !bnd) {
-                    const int row = (S.desc[i] >> 5) & 0xff;
-                    atomicAdd(&S.rowcnt[row >> 2], 1u << (8 * (row & 3)));   // a byte a row: at most 16
-                    if (INDEX) S.nint = 1;
-                }
-            }
-        }
-        __syncthreads();
         const int nb_ = S.nbnd;
         if (FAST && nb_ > BL) {                 // block-uniform; nothing global written yet
             if (tid == 0) W.ovf[atomicAdd(W.novf, 1)] = (int32_t)t;
@@ -600,10 +589,11 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
             W.psize[pid] = S.aux[i] & (AUX_FACE - 1);
             if (INDEX) W.pvotes[pid] = S.votes[i];
             S.aux[i] = -1 - k;                   // from here on: boundary root k
+            atomicAdd(&S.rowcnt[row >> 2], 0u - (1u << (8 * (row & 3))));   // not an interior root
         }
         if (tid == 0)
             W.tinfo[t] = make_int4(g.x0, g.y0, g.z0,
-                                   nb_ | (total << 11) | (lat << 24) | (INDEX && nb_ == 1 && !S.nint ? TILE_ONE_PIECE : 0));
+                                   nb_ | (total << 11) | (lat << 24) | (INDEX && nb_ == 1 && S.nroot == 1 ? TILE_ONE_PIECE : 0));
         __syncthreads();
 
         // interior roots per row segment
@@ -625,7 +615,7 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
             C[i] = c;
         }
 
-        if (INDEX && S.nint) {                    // the tag of each run's piece, as if it were interior
+        if (INDEX && S.nroot > nb_) {             // the tag of each run's piece, as if it were interior
             const int lane = tid & 31;
             uint32_t *T = W.tag + t * (MR / 16);
             for (int i0 = tid - lane; i0 < total; i0 += NT) {
@@ -1488,8 +1478,8 @@ __global__ void __launch_bounds__(256) k_interior_update(const int8_t *prev, con
 
 // Dense form in place: a far site's state stays where it is, so only the groups of four
 // sites that hold a near one are read and written (one in fifty for 729 capsules at
-// 1024^3), and the pass is the read of the index field: 0.97 ms with every state moved,
-// 0.66 ms so.  Four 16-byte index loads in flight a thread.  vec: index 16-byte and state
+// 1024^3), and the pass is the read of the index field: 0.98 ms with every state moved,
+// 0.72 ms so.  Four 16-byte index loads in flight a thread.  vec: index 16-byte and state
 // 4-byte aligned.
 __global__ void __launch_bounds__(256) k_interior_update_in_place(int8_t *state, const float *index, int64_t n,
                                                                    bool vec) {
