@@ -16,6 +16,11 @@
 // Runs are numbered in row-major order of their first sites, so each cluster's root
 // (its smallest run id) holds its smallest site, and ranking roots by run id ranks the
 // clusters by label.  No workspace is used: the results go straight to the outputs.
+//
+// Latency bounds a call (barriers, and chains of dependent shared loads).  With links for
+// the first pairs, ranks from root bits and one scan for two segments a thread, one CTA
+// takes 26.6 us for 32^3 at p = 0.3 (36.9 with every pair united by its segment's thread
+// and ranks by blocks of run ids), a batch of 32 such lattices 29 us (89).
 #include <cooperative_groups.h>
 
 #include <cstddef>
@@ -38,10 +43,14 @@ struct SmallSmem {
     int par[SMALL_MAX_RUNS];           // union-find over run ids; after compression: the root
     int sz[SMALL_MAX_RUNS];            // piece size, summed at each root
     uint16_t desc[SMALL_MAX_RUNS];     // per run: (segment << 5) | first x
+    uint32_t rootbal[SMALL_MAX_RUNS / 32];   // cluster-root bits of each 32 run ids
+    uint16_t rootpre[SMALL_MAX_RUNS / 32];   // roots before them
     int warp_tmp[32];
     int scan_total;
     int hist[32];
 };
+static_assert(SMALL_MAX_RUNS % 32 == 0 && SMALL_MAX_RUNS / 32 <= SNT, "one thread scans one word of root bits");
+static_assert(SMALL_MAX_SEG <= 2 * SNT, "two segments a thread");
 static_assert(SMALL_MAX_SEG <= 2048 && SMALL_MAX_RUNS <= 65535, "desc holds an 11-bit segment, sb a 16-bit run id");
 static_assert(sizeof(SmallSmem) <= 227 * 1024, "one CTA's shared memory");
 
@@ -99,6 +108,7 @@ __global__ void __launch_bounds__(SNT, 1) k_small_label(const __grid_constant__ 
     constexpr int NW = SNT / 32;
     const int nx = L.nx, ny = L.ny, nz = L.nz, nbx = L.nbx;
     const int nseg = nbx * ny * nz;
+    const bool flat = (nx & 31) == 0;   // segment s is sites 32 s .. 32 s + 31 of the lattice
     const FastDiv div_nbx((uint32_t)nbx), div_ny((uint32_t)ny);
     if (tid < 32) S.hist[tid] = 0;
 
@@ -110,8 +120,12 @@ __global__ void __launch_bounds__(SNT, 1) k_small_label(const __grid_constant__ 
 #pragma unroll
         for (int j = 0; j < INF; ++j) {
             const int s = s0 + NW * j;
-            const int q = (int)div_nbx((uint32_t)s), x = (s - q * nbx) * 32 + lane;
-            v[j] = (s < nseg && x < nx) ? __ldg(L.phi + (int64_t)q * nx + x) : 0.0f;
+            if (flat) {
+                v[j] = s < nseg ? __ldg(L.phi + 32 * s + lane) : 0.0f;
+            } else {
+                const int q = (int)div_nbx((uint32_t)s), x = (s - q * nbx) * 32 + lane;
+                v[j] = (s < nseg && x < nx) ? __ldg(L.phi + (int64_t)q * nx + x) : 0.0f;
+            }
         }
 #pragma unroll
         for (int j = 0; j < INF; ++j) {
@@ -121,54 +135,79 @@ __global__ void __launch_bounds__(SNT, 1) k_small_label(const __grid_constant__ 
     }
     __syncthreads();
 
-    // a2: run ids: a scan of the run counts of segments 2t and 2t + 1
-    const int s_a = 2 * tid, s_b = 2 * tid + 1;
-    const int n_a = s_a < nseg ? __popc(run_starts(S.m[s_a])) : 0;
-    const int n_b = s_b < nseg ? __popc(run_starts(S.m[s_b])) : 0;
-    int total;
-    const int base = cta_exscan<SNT>(n_a + n_b, S, total);
-    if (s_a < nseg) S.sb[s_a] = (uint16_t)base;
-    if (s_b < nseg) S.sb[s_b] = (uint16_t)(base + n_a);
+    // a2: run ids: one scan of the run counts of segments t (low half) and t + SNT
+    const uint32_t w_a = tid < nseg ? S.m[tid] : 0u, w_b = tid + SNT < nseg ? S.m[tid + SNT] : 0u;
+    const int n_a = __popc(run_starts(w_a)), n_b = __popc(run_starts(w_b));
+    int packed_total;
+    const int packed = cta_exscan<SNT>(n_a | (n_b << 16), S, packed_total);
+    const int total = (packed_total & 0xffff) + (packed_total >> 16);
+    auto first_run = [&](int h) { return h ? (packed_total & 0xffff) + (packed >> 16) : packed & 0xffff; };
     for (int h = 0; h < 2; ++h) {   // own node and descriptor of every run
-        const int s = 2 * tid + h;
+        const int s = tid + h * SNT;
         if (s >= nseg) break;
-        uint32_t w = run_starts(S.m[s]);
-        int id = base + (h ? n_a : 0);
-        while (w) {
-            const int x0 = __ffs(w) - 1;
-            w &= w - 1;
+        int id = first_run(h);
+        S.sb[s] = (uint16_t)id;
+        for (uint32_t w = run_starts(h ? w_b : w_a); w; ++id) {
+            const uint32_t low = w & (0u - w);
+            w ^= low;
             S.par[id] = id;
             S.sz[id] = 0;
-            S.desc[id] = (uint16_t)((s << 5) | x0);
-            ++id;
+            S.desc[id] = (uint16_t)((s << 5) | top_bit(low));
         }
     }
     __syncthreads();
 
     // a3: unions with the lower neighbours along x (previous segment), y and z, and
     // across the periodic edges (the wrap of an axis of length 1 is a self-edge; one of
-    // length 2 repeats an interior edge)
+    // length 2 repeats an interior edge).  As in the tile pass, a run's first pair with a
+    // lower row is a store into its own node, and a z pair whose site is joined through
+    // its y neighbours is left out; the others are united after a barrier.
+    uint32_t rest_y[2] = {0u, 0u}, rest_z[2] = {0u, 0u};
+    for (int h = 0; h < 2; ++h) {
+        const int s = tid + h * SNT;
+        const uint32_t w = h ? w_b : w_a;
+        if (s >= nseg || !w) continue;
+        const int q = (int)div_nbx((uint32_t)s), z = (int)div_ny((uint32_t)q), y = q - z * ny;
+        const int sy = s - nbx, sz = s - nbx * ny;
+        const uint32_t my = y > 0 ? S.m[sy] : 0u, mz = z > 0 ? S.m[sz] : 0u;
+        const uint32_t oy = w & my, oz = w & mz, uy = fill_up(w, oy);
+        const uint32_t osy = run_starts(oy), osz = run_starts(oz), rs = run_starts(w);
+        const uint32_t ylink = osy & ~(uy << 1);
+        const uint32_t zlink = osz & ~(fill_up(w, oz) << 1) & ~(uy | fill_down(w, oy));
+        rest_y[h] = osy ^ ylink;
+        rest_z[h] = osz & ~zlink;
+        if (y > 0 && z > 0) rest_z[h] &= ~(my & S.m[sz - nbx]);
+        const int b = first_run(h), by = y > 0 ? S.sb[sy] : 0, bz = z > 0 ? S.sb[sz] : 0;
+        const uint32_t rsy = run_starts(my), rsz = run_starts(mz);
+        for (uint32_t link = ylink | zlink; link;) {
+            const uint32_t low = link & (0u - link), le = low | (low - 1u);
+            link ^= low;
+            const bool iy = (my & low) != 0u;
+            S.par[b + __popc(rs & le) - 1] = (iy ? by : bz) + __popc((iy ? rsy : rsz) & le) - 1;
+        }
+    }
+    __syncthreads();
     const int cap = (local_cap > 0 && local_cap < total) ? local_cap : total;
     const int lastbit = (nx - 1) & 31;   // bit of x = nx - 1 in the last segment of a row
-    for (int s = tid; s < nseg; s += SNT) {   // strided: every thread has a segment up to 1024 of them
-        const uint32_t w = S.m[s];
-        if (!w) continue;
-        const int b = S.sb[s];
+    for (int h = 0; h < 2; ++h) {
+        const int s = tid + h * SNT;
+        const uint32_t w = h ? w_b : w_a;
+        if (s >= nseg || !w) continue;
+        const int b = first_run(h);
         const int q = (int)div_nbx((uint32_t)s), bx = s - q * nbx, z = (int)div_ny((uint32_t)q), y = q - z * ny;
-        auto join = [&](int t) {   // every overlap of segment s with segment t
+        auto join = [&](int t, uint32_t os) {   // the pairs of segments s and t that start at bits os
             const uint32_t wt = S.m[t];
-            uint32_t os = run_starts(w & wt);
             const int bt = S.sb[t];
             while (os) {
-                const int x = __ffs(os) - 1;
+                const int x = top_bit(os & (0u - os));
                 os &= os - 1;
                 s_union(S.par, srun(b, w, x), srun(bt, wt, x), cap, status);
             }
         };
-        if (y > 0) join(s - nbx);
-        else if (L.per[1] && ny >= 2) join(s + (ny - 1) * nbx);
-        if (z > 0) join(s - nbx * ny);
-        else if (L.per[2] && nz >= 2) join(s + (nz - 1) * nbx * ny);
+        if (rest_z[h]) join(s - nbx * ny, rest_z[h]);
+        if (rest_y[h]) join(s - nbx, rest_y[h]);
+        if (y == 0 && L.per[1] && ny >= 2) join(s + (ny - 1) * nbx, run_starts(w & S.m[s + (ny - 1) * nbx]));
+        if (z == 0 && L.per[2] && nz >= 2) join(s + (nz - 1) * nbx * ny, run_starts(w & S.m[s + (nz - 1) * nbx * ny]));
         if ((w & 1u) && bx > 0 && (S.m[s - 1] >> 31))
             s_union(S.par, b, srun(S.sb[s - 1], S.m[s - 1], 31), cap, status);
         if ((w & 1u) && bx == 0 && L.per[0] && nx >= 2) {
@@ -178,42 +217,54 @@ __global__ void __launch_bounds__(SNT, 1) k_small_label(const __grid_constant__ 
     }
     __syncthreads();
 
-    // compression and piece sizes
-    for (int i = tid; i < total; i += SNT) {
-        const int root = s_find_ro(S.par, i);
-        S.par[i] = root;
-        const int d = S.desc[i];
-        atomicAdd(&S.sz[root], run_len(S.m[d >> 5], d & 31));
+    // compression (two levels a step), piece sizes, and the root bits of the run ids
+    for (int i0 = wid * 32; i0 < total; i0 += SNT) {
+        const int i = i0 + lane;
+        bool is_root = false;
+        if (i < total) {
+            int root = S.par[i];
+            for (int up = S.par[root]; up != root; up = S.par[root]) root = S.par[up];
+            S.par[i] = root;
+            const int d = S.desc[i];
+            atomicAdd(&S.sz[root], run_len(S.m[d >> 5], d & 31));
+            is_root = root == i;
+        }
+        const uint32_t bal = __ballot_sync(0xffffffffu, is_root);
+        if (lane == 0) S.rootbal[i0 >> 5] = bal;
     }
     __syncthreads();
 
-    // a4, a6, a7: roots in run order get consecutive ranks; each thread takes a
-    // contiguous block of run ids
-    const int per = (total + SNT - 1) / SNT;
-    const int i0 = tid * per, i1 = min(i0 + per, total);
-    int nr = 0;
-    for (int i = i0; i < i1; ++i) nr += S.par[i] == i;
+    // a4, a6, a7: the roots in run order get consecutive ranks (a scan of the words of
+    // root bits), and sizes leave in that order
+    const int nchunks = (total + 31) >> 5;
     int nclus;
-    int rank = cta_exscan<SNT>(nr, S, nclus);
+    const int before = cta_exscan<SNT>(tid < nchunks ? __popc(S.rootbal[tid]) : 0, S, nclus);
+    if (tid < nchunks) S.rootpre[tid] = (uint16_t)before;
+    __syncthreads();
     const int64_t capr = L.sizes_cap;
-    for (int i = i0; i < i1; ++i) {
-        if (S.par[i] != i) continue;
+    for (int i0 = wid * 32; i0 < total; i0 += SNT) {
+        const uint32_t bal = S.rootbal[i0 >> 5];
+        if (!((bal >> lane) & 1u)) continue;
+        const int i = i0 + lane, rank = S.rootpre[i0 >> 5] + __popc(bal & ((1u << lane) - 1u));
         const int size = S.sz[i];
         if (rank < capr) L.sizes[rank] = size;
-        ++rank;
-        atomicAdd(&S.hist[31 - __clz(size)], 1);
+        atomicAdd(&S.hist[top_bit((uint32_t)size)], 1);
         const int d = S.desc[i], rs_ = d >> 5, rq = (int)div_nbx((uint32_t)rs_);
         S.sz[i] = rq * nx + (rs_ - rq * nbx) * 32 + (d & 31);   // from here on: the root's site (its label)
     }
     __syncthreads();
 
     // a5: labels, one warp per segment, one lane per site
+#pragma unroll 4
     for (int s = wid; s < nseg; s += NW) {
-        const int q = (int)div_nbx((uint32_t)s), x = (s - q * nbx) * 32 + lane;
-        if (x >= nx) continue;
         const uint32_t w = S.m[s];
         const int lab = ((w >> lane) & 1u) ? S.sz[S.par[srun(S.sb[s], w, lane)]] : -1;
-        L.labels[(int64_t)q * nx + x] = lab;
+        if (flat) {
+            L.labels[32 * s + lane] = lab;
+        } else {
+            const int q = (int)div_nbx((uint32_t)s), x = (s - q * nbx) * 32 + lane;
+            if (x < nx) L.labels[(int64_t)q * nx + x] = lab;
+        }
     }
     __syncthreads();
     if (tid < 32 && L.hist) L.hist[tid] = S.hist[tid];
