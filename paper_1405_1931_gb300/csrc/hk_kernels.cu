@@ -242,8 +242,8 @@ __global__ void __launch_bounds__(256) k_occupancy_tma(const __grid_constant__ T
 //
 // Bound by instruction issue (90 % of its rate): 2 warp instructions a site at p_c.  With
 // most pairs linked or left out instead of united, and with boundary pieces listed by the
-// run that first touches a face instead of in passes over all runs: 1.93 against 2.38 ms
-// at 1024^3, p_c, 0.81 against 1.06 ms on blocks of 16^3, 0.127 against 0.148 ms on a
+// run that first touches a face instead of in passes over all runs: 1.90 against 2.38 ms
+// at 1024^3, p_c, 0.80 against 1.06 ms on blocks of 16^3, 0.127 against 0.148 ms on a
 // 512^3 bijel.
 // --------------------------------------------------------------------------------------
 template <int TY, int TZ, int CAP, int BL, bool INDEX>
@@ -503,17 +503,18 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
         // roots of each row are counted, a byte a row (at most 16).
         for (int i = tid; i < total; i += NT) {
             int root = S.par[i];
-            for (int up = S.par[root]; up != root; up = S.par[root]) root = S.par[up];   // two levels a step
+            while (true) {                       // two levels a step
+                const int up = S.par[root];
+                root = S.par[up];
+                if (root == up) break;
+            }
             S.par[i] = root;
             const int d = S.desc[i], row = (d >> 5) & 0xff;
             const int len = run_len(S.m[row], d & 31);
-            if (d & DESC_TOUCH) {
-                if (atomicAdd(&S.aux[root], len + AUX_FACE) < AUX_FACE) {
-                    const int k = atomicAdd(&S.nbnd, 1);
-                    if (k < BL) S.blist[k] = (uint16_t)root;
-                }
-            } else {
-                atomicAdd(&S.aux[root], len);
+            const int face = (d & DESC_TOUCH) ? AUX_FACE : 0;
+            if (atomicAdd(&S.aux[root], len + face) + (AUX_FACE - face) < AUX_FACE) {
+                const int k = atomicAdd(&S.nbnd, 1);
+                if (k < BL) S.blist[k] = (uint16_t)root;
             }
             if (root == i) {
                 atomicAdd(&S.rowcnt[row >> 2], 1u << (8 * (row & 3)));
