@@ -283,6 +283,11 @@ __global__ void __launch_bounds__(SNT, 1) k_small_label(const __grid_constant__ 
 // root then learns its cluster root, so each run reaches its root in two steps, and
 // each run's label is resolved once per run, not per site.  The phases that reach other
 // CTAs are separated by cluster barriers.
+//
+// Latency bounds a call here too.  A 32^3 lattice gives a CTA 64 segments, so the pairs
+// inside a CTA that links do not take are shared out by eighths of a segment: 20.6 us at
+// p = 0.3 and 22.5 at 0.45 (24.5 and 24.6 with all pairs counted, listed and united; 22.9
+// and 26.7 with one thread a segment).
 // ---------------------------------------------------------------------------------------
 // CTAs per lattice: 16 where the device co-schedules that many (a non-portable cluster
 // size), else 8 (the portable size); a template parameter of the kernel (CSB = log2).
@@ -291,7 +296,7 @@ constexpr int CSEG = 1024;         // row segments per CTA
 constexpr int CRUN_BITS = 14;
 constexpr int CRUN = 1 << CRUN_BITS;   // runs per CTA: at most 16 per segment
 constexpr int DESC_LROOT = 0x8000;     // desc flag: the run is the root of its CTA-local tree
-static_assert(16 * CSEG <= CRUN && CSEG <= 2 * CNT, "run ids of a CTA; two segments per thread in the scan");
+static_assert(16 * CSEG <= CRUN && CSEG <= CNT, "run ids of a CTA; one segment per thread in the union rounds");
 
 struct ClusterSmem {
     uint32_t m[CSEG];        // occupancy word of each of this CTA's row segments
@@ -462,9 +467,9 @@ __global__ void __cluster_dims__(1 << CSB, 1, 1) __launch_bounds__(CNT, 1)
     // edges, in two rounds.  First the edges inside this CTA, on local run ids in its own
     // shared memory; then, once every CTA has compressed its runs onto their local roots,
     // the edges to runs of other CTAs, joined between local roots through distributed
-    // shared memory.  Each round lists its run pairs first (a scan of per-segment counts;
-    // sz serves as the list), so that the unions spread over all threads; a round whose
-    // list would not fit joins each segment's pairs where they are found.
+    // shared memory.  The second round lists its run pairs first (a scan of per-segment
+    // counts; sz serves as the list), so that the unions spread over all threads; where
+    // the list would not fit each segment's pairs are joined as they are found.
     const int lastbit = (nx - 1) & 31;
     auto neighbours = [&](int ls, auto &&edge) {   // edge(global segment t) for every lower neighbour
         const int sg = seg0 + ls;
@@ -479,65 +484,149 @@ __global__ void __cluster_dims__(1 << CSB, 1, 1) __launch_bounds__(CNT, 1)
         lt = t - o * rp * nbx;
         return o;
     };
-    // every pair of runs joined by an edge of segment ls: pair(own local run, CTA, its run)
-    auto pairs = [&](int ls, bool cross, auto &&pair) {
+    // every pair of runs joined by an edge of segment ls to another CTA: pair(own local run,
+    // CTA, its run)
+    auto pairs = [&](int ls, auto &&pair) {
         const uint32_t w = S.m[ls];
         if (!w) return;
         const int b = S.sb[ls];
         neighbours(ls, [&](int t) {
             int lt;
             const int o = owner(t, lt);
-            if ((o != c) != cross) return;
-            const uint32_t wt = o == c ? S.m[lt] : *cl.map_shared_rank(&S.m[lt], o);
+            if (o == c) return;
+            const uint32_t wt = *cl.map_shared_rank(&S.m[lt], o);
             uint32_t os = run_starts(w & wt);
             if (!os) return;
-            const int bt = o == c ? S.sb[lt] : *cl.map_shared_rank(&S.sb[lt], o);
+            const int bt = *cl.map_shared_rank(&S.sb[lt], o);
             while (os) {
                 const int x = __ffs(os) - 1;
                 os &= os - 1;
                 pair(srun(b, w, x), o, srun(bt, wt, x));
             }
         });
-        if (cross) return;
-        const int bx = (seg0 + ls) - (int)div_nbx((uint32_t)(seg0 + ls)) * nbx;   // a row lives in one CTA
-        if ((w & 1u) && bx > 0 && (S.m[ls - 1] >> 31)) pair(b, c, srun(S.sb[ls - 1], S.m[ls - 1], 31));
-        if ((w & 1u) && bx == 0 && L.per[0] && nx >= 2) {
-            const int t = ls + nbx - 1;
-            if ((S.m[t] >> lastbit) & 1u) pair(b, c, srun(S.sb[t], S.m[t], lastbit));
-        }
     };
-    // one round: count, list and join the pairs of this thread's segments (2t, 2t + 1)
-    auto round = [&](bool cross, auto &&join) {
+    // count, list and join them, one segment a thread
+    auto join_cross = [&](auto &&join) {
         int np = 0;
-        for (int h = 0; h < 2; ++h)
-            if (2 * tid + h < nseg) pairs(2 * tid + h, cross, [&](int, int, int) { ++np; });
+        if (tid < nseg) pairs(tid, [&](int, int, int) { ++np; });
         int npairs;
         int j = cta_exscan<CNT>(np, S, npairs);
         if (npairs <= CRUN) {
-            for (int h = 0; h < 2; ++h)
-                if (2 * tid + h < nseg)
-                    pairs(2 * tid + h, cross, [&](int a, int o, int bb) {
-                        S.sz[j++] = (int)(((uint32_t)a << (CRUN_BITS + CS_BITS)) | ((uint32_t)o << CRUN_BITS) |
-                                          (uint32_t)bb);
-                    });
+            if (tid < nseg)
+                pairs(tid, [&](int a, int o, int bb) {
+                    S.sz[j++] = (int)(((uint32_t)a << (CRUN_BITS + CS_BITS)) | ((uint32_t)o << CRUN_BITS) |
+                                      (uint32_t)bb);
+                });
             __syncthreads();
             for (int k = tid; k < npairs; k += CNT) {
-                const int v = S.sz[k];
-                const uint32_t u = (uint32_t)v;
+                const uint32_t u = (uint32_t)S.sz[k];
                 join((int)(u >> (CRUN_BITS + CS_BITS)), (int)((u >> CRUN_BITS) & (CS - 1)), (int)(u & (CRUN - 1)));
             }
-        } else {
-            for (int h = 0; h < 2; ++h)
-                if (2 * tid + h < nseg) pairs(2 * tid + h, cross, join);
+        } else if (tid < nseg) {
+            pairs(tid, join);
         }
     };
     static_assert(2 * CRUN_BITS + CS_BITS <= 32 && CS <= 32, "a listed pair packs into 32 bits");
     {
         const int lcap = (local_cap > 0 && local_cap < total) ? local_cap : total;
-        round(false, [&](int a, int, int bb) { s_union(S.par, a, bb, lcap, status); });
+        // the edges inside the CTA, one segment a thread: as in the tile pass a run's first
+        // pair with a lower row is a store into its own node and a z pair whose site is
+        // joined through its y neighbours is left out; the others follow after a
+        // barrier, eight shares a segment (a byte of its z or y pairs and some of its edges)
+        // over as many threads as there are
+        // (from half as many segments as threads on: all listed by a scan and taken in turn,
+        // 51 against 54 us at 64 x 96 x 80, p_c)
+        const int row = nbx * ny;
+        uint32_t osy = 0, osz = 0;
+        if (tid < nseg) {
+            const int ls = tid, q = (int)div_nbx((uint32_t)(seg0 + ls)), z = (int)div_ny((uint32_t)q), y = q - z * ny;
+            const uint32_t w = S.m[ls];
+            const uint32_t my = y > 0 && ls >= nbx ? S.m[ls - nbx] : 0u, mz = z > 0 && ls >= row ? S.m[ls - row] : 0u;
+            const uint32_t oy = w & my, oz = w & mz, uy = fill_up(w, oy), rs = run_starts(w);
+            osy = run_starts(oy);
+            osz = run_starts(oz);
+            const uint32_t ylink = osy & ~(uy << 1);
+            const uint32_t zlink = osz & ~(fill_up(w, oz) << 1) & ~(uy | fill_down(w, oy));
+            osy ^= ylink;
+            osz &= ~zlink;
+            if (my && mz && ls >= row + nbx) osz &= ~(my & S.m[ls - row - nbx]);
+            const uint32_t rsy = run_starts(my), rsz = run_starts(mz);
+            const int b = S.sb[ls], by = my ? S.sb[ls - nbx] : 0, bz = mz ? S.sb[ls - row] : 0;
+            for (uint32_t link = ylink | zlink; link;) {
+                const uint32_t low = link & (0u - link), le = low | (low - 1u);
+                link ^= low;
+                const bool iy = (my & low) != 0u;
+                S.par[b + __popc(rs & le) - 1] = (iy ? by : bz) + __popc((iy ? rsy : rsz) & le) - 1;
+            }
+        }
+        bool listed = false;                         // CTA-uniform
+        if (2 * nseg >= CNT) {
+            int npairs;
+            int j = cta_exscan<CNT>(__popc(osz) + __popc(osy), S, npairs);   // ends with a barrier: links are done
+            listed = npairs <= CRUN;
+            if (listed) {
+                auto list = [&](int t, uint32_t os) {
+                    if (!os) return;
+                    const uint32_t w = S.m[tid], wt = S.m[t];
+                    const int b = S.sb[tid], bt = S.sb[t];
+                    for (; os; os &= os - 1u) {
+                        const int x = top_bit(os & (0u - os));
+                        S.sz[j++] = (srun(b, w, x) << CRUN_BITS) | srun(bt, wt, x);
+                    }
+                };
+                list(tid - row, osz);
+                list(tid - nbx, osy);
+                __syncthreads();
+                for (int k = tid; k < npairs; k += CNT)
+                    s_union(S.par, S.sz[k] >> CRUN_BITS, S.sz[k] & (CRUN - 1), lcap, status);
+            }
+        }
+        if (!listed && tid < nseg) {
+            S.sz[tid] = (int)osz;
+            S.sz[CSEG + tid] = (int)osy;
+        }
+        __syncthreads();
+        const int groups = nseg > 0 ? CNT / nseg : 1, group = nseg > 0 ? tid / nseg : CNT;
+        for (int share = (listed ? 4 : 0) + group; group < groups && share < 8; share += groups) {
+            const int ls = tid - group * nseg;
+            const uint32_t w = S.m[ls];
+            if (!w) continue;
+            const int b = S.sb[ls];
+            auto join = [&](int t, uint32_t os) {   // the pairs of segments ls and t that start at bits os
+                if (!os) return;
+                const uint32_t wt = S.m[t];
+                const int bt = S.sb[t];
+                for (; os; os &= os - 1u) {
+                    const int x = top_bit(os & (0u - os));
+                    s_union(S.par, srun(b, w, x), srun(bt, wt, x), lcap, status);
+                }
+            };
+            const uint32_t part = 0xffu << (8 * (share & 3));
+            if (!listed) {
+                if (share < 4) join(ls - row, (uint32_t)S.sz[ls] & part);
+                else join(ls - nbx, (uint32_t)S.sz[CSEG + ls] & part);
+            }
+            if (share >= 4 && share < 7) {           // periodic edges and rows of several segments
+                const int q = (int)div_nbx((uint32_t)(seg0 + ls)), bx = seg0 + ls - q * nbx, z = (int)div_ny((uint32_t)q);
+                const int y = q - z * ny, wy = ls + (ny - 1) * nbx, wz = ls + (nz - 1) * row;
+                if (share == 4 && y == 0 && L.per[1] && ny >= 2 && wy < nseg) join(wy, run_starts(w & S.m[wy]));
+                if (share == 5 && z == 0 && L.per[2] && nz >= 2 && wz < nseg) join(wz, run_starts(w & S.m[wz]));
+                if (share == 6 && (w & 1u)) {
+                    if (bx > 0 && (S.m[ls - 1] >> 31)) s_union(S.par, b, srun(S.sb[ls - 1], S.m[ls - 1], 31), lcap, status);
+                    if (bx == 0 && L.per[0] && nx >= 2) {
+                        const int t = ls + nbx - 1;
+                        if ((S.m[t] >> lastbit) & 1u) s_union(S.par, b, srun(S.sb[t], S.m[t], lastbit), lcap, status);
+                    }
+                }
+            }
+        }
         __syncthreads();
         // local roots, then cluster numbers: every run points at its local root
-        for (int i = tid; i < total; i += CNT) S.sz[i] = s_find_ro(S.par, i);
+        for (int i = tid; i < total; i += CNT) {
+            int root = S.par[i];
+            for (int up = S.par[root]; up != root; up = S.par[root]) root = S.par[up];   // two levels a step
+            S.sz[i] = root;
+        }
         __syncthreads();
         for (int i = tid; i < total; i += CNT) {
             const int r = S.sz[i];
@@ -548,7 +637,7 @@ __global__ void __cluster_dims__(1 << CSB, 1, 1) __launch_bounds__(CNT, 1)
     cl.sync();
     {   // the edges to other CTAs, joined between the two runs' local roots
         const int cap = (local_cap > 0 && local_cap < CS * CRUN) ? local_cap : CS * CRUN;
-        round(true, [&](int a, int o, int bb) {
+        join_cross([&](int a, int o, int bb) {
             V.unite(S.par[a], *cl.map_shared_rank(&S.par[bb], o), cap, status);
         });
     }
