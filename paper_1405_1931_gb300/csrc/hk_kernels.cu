@@ -1477,32 +1477,50 @@ __global__ void __launch_bounds__(256) k_interior_update(const int8_t *prev, con
     }
 }
 
-// Dense form in place: a far site's state stays where it is, so only the groups of four
-// sites that hold a near one are read and written (one in fifty for 729 capsules at
-// 1024^3), and the pass is the read of the index field: 0.98 ms with every state moved,
-// 0.72 ms so.  Four 16-byte index loads in flight a thread.  vec: index 16-byte and state
-// 4-byte aligned.
-__global__ void __launch_bounds__(256) k_interior_update_in_place(int8_t *state, const float *index, int64_t n,
+// Dense form in place: a far site's state stays where it is, so only the 32-byte sectors of
+// states (32 sites, two lanes) that hold a near one are read and written, and away from
+// membranes the pass is the read of the index field: 729 capsules at 1024^3, 0.74 against
+// 0.98 ms with every state moved.  A warp half of whose sectors held one loads its next
+// states along with the index values, so that fields full of near sites lose little (0.32
+// against 0.30 ms for 343 M sites, a third of them near; 0.30 with a twentieth near).
+// Groups of four sites, read and written one by one, were faster on the capsules (0.71
+// ms) and slower on fuller fields (0.35 and 0.42 ms).  vec: both arrays 16-byte aligned.
+__global__ void __launch_bounds__(256, 8) k_interior_update_in_place(int8_t *state, const float *index, int64_t n,
                                                                    bool vec) {
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
     int64_t done = 0;
     if (vec) {
-        constexpr int U = 4;
-        const int64_t nv = n / 4;
-        for (int64_t i0 = t0; i0 < nv; i0 += U * stride) {
-            float4 v[U];
+        const int64_t nv = n / 16, lane = threadIdx.x & 31;
+        bool many = false;                             // warp-uniform
+        for (int64_t i0 = t0 - lane; i0 < nv; i0 += stride) {
+            const int64_t i = i0 + lane;
+            const bool in = i < nv;
+            int4 sp = make_int4(0, 0, 0, 0);
+            if (many && in) sp = __ldcs(reinterpret_cast<const int4 *>(state) + i);
+            float4 v[4];
 #pragma unroll
-            for (int u = 0; u < U; ++u)
-                v[u] = i0 + u * stride < nv ? __ldcs(reinterpret_cast<const float4 *>(index) + i0 + u * stride)
-                                            : make_float4(-1.f, -1.f, -1.f, -1.f);
+            for (int q = 0; q < 4; ++q)
+                v[q] = in ? __ldcs(reinterpret_cast<const float4 *>(index) + 4 * i + q) : make_float4(-1.f, -1.f, -1.f, -1.f);
+            bool near = false;
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                if (v[u].x < -0.5f && v[u].y < -0.5f && v[u].z < -0.5f && v[u].w < -0.5f) continue;
-                uint32_t *p = reinterpret_cast<uint32_t *>(state) + i0 + u * stride;
-                *p = update_byte(update_byte(update_byte(update_byte(*p, 0, v[u].x), 1, v[u].y), 2, v[u].z), 3, v[u].w);
+            for (int q = 0; q < 4; ++q)
+                near |= !(v[q].x < -0.5f && v[q].y < -0.5f && v[q].z < -0.5f && v[q].w < -0.5f);
+            const uint32_t nb = __ballot_sync(0xffffffffu, near);
+            if (in && ((nb >> (lane & ~1)) & 3u)) {    // this lane's sector holds a near site
+                if (!many) sp = __ldcs(reinterpret_cast<const int4 *>(state) + i);
+                uint32_t w[4] = {(uint32_t)sp.x, (uint32_t)sp.y, (uint32_t)sp.z, (uint32_t)sp.w};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    w[q] = update_byte(w[q], 0, v[q].x);
+                    w[q] = update_byte(w[q], 1, v[q].y);
+                    w[q] = update_byte(w[q], 2, v[q].z);
+                    w[q] = update_byte(w[q], 3, v[q].w);
+                }
+                __stcs(reinterpret_cast<int4 *>(state) + i, make_int4((int)w[0], (int)w[1], (int)w[2], (int)w[3]));
             }
+            many = __popc((nb | (nb >> 1)) & 0x55555555u) >= 8;
         }
-        done = nv * 4;
+        done = nv * 16;
     }
     for (int64_t s = done + t0; s < n; s += stride) {
         const float v = index[s];
@@ -1530,10 +1548,14 @@ static unsigned stream_grid(int64_t units) {
     return (unsigned)(g > 0 ? g : 1);
 }
 
+// In place, from this many sites on, only the states near a membrane are moved.  Below, both
+// arrays stay in L2 between steps and reading the states first is as fast or faster (12.3
+// against 14.4 us at 256^3); above, it is not (42.6 against 58.4 us at 400^3).
+constexpr int64_t UPDATE_IN_PLACE_MIN = (int64_t)1 << 25;
 cudaError_t launch_interior_update(const int8_t *prev, const float *index, int64_t n, int8_t *out, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    if (prev == out) {
-        const bool vec = (reinterpret_cast<uintptr_t>(index) & 15) == 0 && (reinterpret_cast<uintptr_t>(out) & 3) == 0;
+    if (prev == out && n >= UPDATE_IN_PLACE_MIN) {
+        const bool vec = ((reinterpret_cast<uintptr_t>(index) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
         k_interior_update_in_place<<<stream_grid(vec ? n / 16 + 1 : n), 256, 0, st>>>(out, index, n, vec);
         return cudaGetLastError();
     }

@@ -28,3 +28,23 @@ def test_in_place(n, density):
             got = state.cpu().numpy()
             np.testing.assert_array_equal(got[off_s:off_s + n], want)
             assert (got[:off_s] == 9).all() and (got[off_s + n:] == 9).all()
+
+
+@pytest.mark.parametrize("off_i,off_s", [(0, 0), (1, 0), (0, 4)])
+def test_in_place_large(off_i, off_s):
+    """From 2^25 sites on, with stretches full of near sites, sparse ones and a ragged end."""
+    n = (1 << 25) + 45
+    rng = np.random.default_rng(off_i + off_s)
+    density = np.repeat(rng.choice([0.0, 0.01, 0.3, 1.0], size=n // 5000 + 1), 5000)[:n]
+    I = np.where(rng.random(n, dtype=np.float32) < density, np.where(rng.random(n) < 0.5, -0.25, 0.25), -1.0)
+    I = I.astype(np.float32)
+    prev = rng.integers(-1, 2, size=n).astype(np.int8)
+    want = oracle.interior_update(prev.reshape(1, 1, n), I.reshape(1, 1, n)).reshape(-1)
+    index = torch.full((n + 8,), 0.25, device="cuda")
+    state = torch.full((n + 16,), 9, dtype=torch.int8, device="cuda")
+    index[off_i:off_i + n] = torch.from_numpy(I).cuda()
+    state[off_s:off_s + n] = torch.from_numpy(prev).cuda()
+    hk.interior_update(state[off_s:off_s + n], index[off_i:off_i + n])
+    got = state.cpu().numpy()
+    np.testing.assert_array_equal(got[off_s:off_s + n], want)
+    assert (got[:off_s] == 9).all() and (got[off_s + n:] == 9).all()
