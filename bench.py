@@ -33,8 +33,8 @@ METRIC = "Gsites/s labelled+sized at 1024^3 p_c; batched vs per-lattice; p50/p99
 P_C = 0.3116
 L_HEADLINE = 1024
 # kernels of one hk_label call: occupancy, tile_label (fast pass and the pass over
-# dense tiles), face_merge, piece_finalize, three scan kernels, lattice_finish, flatten
-LAUNCHES_PER_CALL = 10
+# dense tiles), face_merge, piece_finalize, two scan kernels, flatten
+LAUNCHES_PER_CALL = 8
 
 
 def parse():

@@ -113,9 +113,8 @@ int hk_label(hk_ctx *ctx, const float *phi, int nx, int ny, int nz, const int pe
  * votes with the sign of I at the near site (I == 0 and NaN do not vote); more
  * negative votes -> interior, more positive -> exterior, a tie -> -1.
  * Same stream and capacity rules as hk_label; the tags of clusters beyond
- * sizes_cap are not written.  The workspace grows by N/4 bytes (a word of root
- * sites and a rank prefix per 32-site row segment) and 4 B per sizes_cap entry
- * for the votes.
+ * sizes_cap are not written.  The workspace grows by about N bytes (two sign
+ * words per 32 sites, and votes and tags per piece), whatever sizes_cap is.
  * Errors: HK_ERR_ARG, HK_ERR_TOO_LARGE, HK_ERR_NOMEM, HK_ERR_CUDA, HK_ERR_CAPACITY. */
 int hk_label_interior(hk_ctx *ctx, const float *index, int nx, int ny, int nz, const int periodic[3],
                       int32_t *labels_out, int64_t *sizes_out, int64_t sizes_cap,
@@ -333,8 +332,8 @@ int hk_rc_histogram(const int64_t *sizes, const int64_t *n_clusters, int64_t siz
  *              exterior, -1 undetermined); a near site (any other value, NaN
  *              included) the side its value names, 1 for I < 0 and 0 otherwise.
  * This is the full identification the paper uses to initialise the field and to
- * refresh it from time to time.  The clusters' labels, sizes and tags live in
- * the context (about 8.5 bytes a site, grown on demand).  Asynchronous on `stream`.
+ * refresh it from time to time.  It uses the workspace of hk_label_interior and
+ * keeps no labels or sizes.  Asynchronous on `stream`.
  * Errors: HK_ERR_ARG, HK_ERR_TOO_LARGE, HK_ERR_NOMEM, HK_ERR_CUDA. */
 int hk_interior_state(hk_ctx *ctx, const float *index, int nx, int ny, int nz, const int periodic[3],
                       int8_t *state_out, void *stream);
@@ -414,8 +413,9 @@ int hk_set_small_path(hk_ctx *ctx, int enable);
  * set).  hk_get_timing synchronises on the timed calls still in flight and
  * writes up to max_n per-pass AVERAGE durations in milliseconds over all timed
  * calls since timing was enabled to ms_out (host), in pass order: occupancy,
- * tile_label, face_merge, piece_finalize, scan (three kernels), lattice_finish,
- * flatten;
+ * tile_label, face_merge, piece_finalize, scan, lattice_finish (counts and
+ * histograms; no kernel of its own, so about zero), flatten (for
+ * hk_interior_state the pass that writes the states, with scan at zero);
  * *n_out gets the number of passes.  For a batch split into several launch
  * chunks each chunk counts as one call.  Timing adds event records only;
  * results are unchanged.  Errors: HK_ERR_ARG (no timed call yet, NULL ctx or

@@ -296,17 +296,6 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
 // union's retry loop is the one that depends on other threads, and it keeps an
 // explicit bound.
 
-// read-only find: used by compression, where finds run while others store final
-// roots (a halving store there could overwrite a final root with an ancestor)
-__device__ __forceinline__ int s_find_ro(const int *par, int x) {
-    int p = par[x];
-    while (p != x) {
-        x = p;
-        p = par[x];
-    }
-    return x;
-}
-
 // find with path splitting (during the unions): every node passed is pointed at its
 // grandparent, an ancestor, so concurrent finds and links stay valid
 __device__ __forceinline__ int s_find(int *par, int x) {
@@ -419,18 +408,6 @@ __device__ __forceinline__ int block_exscan(int v, int *warp_tmp, int &total) {
 // piece holding the cluster's smallest site index.  The parent array is kept at
 // 4 bytes a piece: finds hop across the whole table, so its footprint in L2 matters.
 // A path visits distinct pieces, so `cap` (the piece-table size) bounds it.
-__device__ __forceinline__ int g_find(int32_t *parent, int x, int64_t cap, int32_t *status) {
-    int p = __ldcg(parent + x);
-    for (int64_t it = 0; p != x; ++it) {
-        if (it > cap) { atomicOr(status, STATUS_GLOBAL_LOOP); return x; }
-        int gp = __ldcg(parent + p);
-        if (gp == p) return p;
-        __stcg(parent + x, gp);    // path halving
-        x = gp;
-        p = __ldcg(parent + x);
-    }
-    return x;
-}
 
 // Read-only find for the compression pass: no halving writes, so the one store
 // each thread makes afterwards (parent[pid] = root) cannot be overwritten by
