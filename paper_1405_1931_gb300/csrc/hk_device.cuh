@@ -227,7 +227,19 @@ __device__ __forceinline__ int top_bit(uint32_t w) {
     return p;
 }
 // bits 0..x set
-__device__ __forceinline__ uint32_t le_mask(int x) { return (2u << x) - 1u; }
+__host__ __device__ __forceinline__ uint32_t le_mask(int x) { return (2u << x) - 1u; }
+// label of site x of a row (occupancy word m, run starts rs, first run id first): its run's
+// entry of lab, or -1 on the medium, where lab is not read -- before the row's first run there
+// is no entry that belongs to it, and before the tile's first none at all
+template <class Lab>
+__host__ __device__ __forceinline__ int site_label(uint32_t m, uint32_t rs, int first, uint32_t le, const Lab &lab) {
+#ifdef __CUDA_ARCH__
+    const int k = __popc(rs & le);
+#else
+    const int k = __builtin_popcount(rs & le);
+#endif
+    return m & (le ^ (le >> 1)) ? lab[first - 1 + k] : -1;
+}
 // run id (within the tile) of occupied site x of a row with run starts rs
 __device__ __forceinline__ int run_of(int rbase, uint32_t rs, int x) { return rbase + __popc(rs & le_mask(x)) - 1; }
 // length of the run starting at bit x0 of m: the first run end at or above x0, which

@@ -1327,15 +1327,13 @@ k_flatten(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles, uint32
                     __stcs(reinterpret_cast<int4 *>(out), v);
                 }
         } else if (ti.x + lane < L.nx) {
-            const uint32_t le = le_mask(lane), me = 1u << lane;
+            const uint32_t le = le_mask(lane);
             for (int yy = wid; yy < TY && ti.y + yy < L.ny; yy += NW) {
                 int32_t *out = L.labels + (int64_t)ti.z * sxy + (int64_t)(ti.y + yy) * L.nx + ti.x + lane;
-#pragma unroll 4
+#pragma unroll 2
                 for (int row = yy; row < nrow; row += TY, out += sxy) {
                     const uint4 w = S.row[row];
-                    int v = S.lab[(int)w.z - 1 + __popc(w.y & le)];
-                    if (!(w.x & me)) v = -1;
-                    __stcs(out, v);
+                    __stcs(out, site_label(w.x, w.y, (int)w.z, le, S.lab));
                 }
             }
         }
