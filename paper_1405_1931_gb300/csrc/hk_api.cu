@@ -20,7 +20,7 @@ using hk::Work;
 
 namespace hk {
 
-Work bind_work(char *base, const Layout &Ly, int32_t *status, int64_t piece_cap, int64_t loop_cap) {
+Work bind_work(char *base, const Layout &Ly, int32_t *status, const Plan &P, int64_t loop_cap) {
     Work W;
     W.mask = reinterpret_cast<uint32_t *>(base + Ly.mask);
     W.codes = reinterpret_cast<uint16_t *>(base + Ly.codes);
@@ -41,7 +41,8 @@ Work bind_work(char *base, const Layout &Ly, int32_t *status, int64_t piece_cap,
     W.pvotes = reinterpret_cast<int32_t *>(base + Ly.pvotes);
     W.tag = reinterpret_cast<uint32_t *>(base + Ly.tag);
     W.novf = status + 1;
-    W.piece_cap = (loop_cap > 0 && loop_cap < piece_cap) ? loop_cap : piece_cap;
+    W.piece_cap = (loop_cap > 0 && loop_cap < P.piece_cap) ? loop_cap : P.piece_cap;
+    W.piece_stride = P.piece_stride;
     W.local_cap = (loop_cap > 0 && loop_cap < INT32_MAX) ? (int32_t)loop_cap : 0;
     W.site_off = 0;
     W.roots = nullptr;
@@ -328,14 +329,15 @@ int run_lattices(hk_ctx *ctx, const hk_lattice *lats, int n, cudaStream_t st, bo
     }
 
     // Launch chunks: at most MAX_LAT_PER_LAUNCH lattices, and few enough tiles that
-    // every piece id (tile * max_boundary + k) and every root count fits in 31 bits.
-    const int64_t max_tiles = ((int64_t)1 << 31) / ti.max_boundary - 1;
+    // every piece id (tile * stride + k) and every root count fits in 31 bits; a lattice that
+    // has more tiles on its own makes a chunk with its own stride (plan_pieces).
+    const int64_t max_tiles = hk::MAX_PIECES / ti.max_boundary - 1;
     std::vector<int> chunk_start;
     {
         int c0 = 0;
         while (c0 < n) {
             chunk_start.push_back(c0);
-            Plan P{0, 0, 0, 0};
+            Plan P{};
             int c1 = c0;
             while (c1 < n && c1 - c0 < hk::MAX_LAT_PER_LAUNCH) {
                 Plan Q = P;
@@ -351,9 +353,10 @@ int run_lattices(hk_ctx *ctx, const hk_lattice *lats, int n, cudaStream_t st, bo
     // size the workspace for the largest chunk
     size_t need = 0;
     for (size_t c = 0; c + 1 < chunk_start.size(); ++c) {
-        Plan P{0, 0, 0, 0};
+        Plan P{};
         for (int i = chunk_start[c]; i < chunk_start[c + 1]; ++i) add_lattice(ti, lats[i].nx, lats[i].ny, lats[i].nz, P);
-        P.piece_cap = P.ntiles * ti.max_boundary;
+        const hk_lattice &l = lats[chunk_start[c]];
+        if (!hk::plan_pieces(ti, P, l.nx, l.ny, l.nz)) return HK_ERR_TOO_LARGE;   // nothing is enqueued yet
         need = std::max(need, hk::make_layout(ti, P, inside || state).total);
     }
     int rc = ensure_ws(ctx, need);
@@ -366,7 +369,7 @@ int run_lattices(hk_ctx *ctx, const hk_lattice *lats, int n, cudaStream_t st, bo
     for (size_t c = 0; c + 1 < chunk_start.size(); ++c) {
         const int c0 = chunk_start[c];
         const int cn = chunk_start[c + 1] - c0;
-        Plan P{0, 0, 0, 0};
+        Plan P{};
         std::vector<LatDev> dev(cn);
         for (int i = 0; i < cn; ++i) {
             const hk_lattice &l = lats[c0 + i];
@@ -390,10 +393,10 @@ int run_lattices(hk_ctx *ctx, const hk_lattice *lats, int n, cudaStream_t st, bo
             d.inside = inside;
             add_lattice(ti, l.nx, l.ny, l.nz, P);
         }
-        P.piece_cap = P.ntiles * ti.max_boundary;
+        hk::plan_pieces(ti, P, lats[c0].nx, lats[c0].ny, lats[c0].nz);
         const hk::Layout Ly = hk::make_layout(ti, P, inside || state);
         char *base = static_cast<char *>(ctx->ws);
-        Work W = hk::bind_work(base, Ly, ctx->dstatus, P.piece_cap, ctx->loop_cap);
+        Work W = hk::bind_work(base, Ly, ctx->dstatus, P, ctx->loop_cap);
         if (!inside && !state) {
             W.neg = W.pos = W.near_tile = W.tag = nullptr;
             W.pvotes = nullptr;
@@ -566,9 +569,9 @@ size_t hk_workspace_bytes(int nx, int ny, int nz) {
     if (nx < 1 || ny < 1 || nz < 1 || (int64_t)nx * ny * nz >= MAX_SITES) return 0;
     TileInfo ti;
     hk::tile_info(DEFAULT_TY, DEFAULT_TZ, ti);
-    Plan P{0, 0, 0, 0};
+    Plan P{};
     add_lattice(ti, nx, ny, nz, P);
-    P.piece_cap = P.ntiles * ti.max_boundary;
+    hk::plan_pieces(ti, P, nx, ny, nz);
     return hk::make_layout(ti, P).total;
 }
 

@@ -69,11 +69,11 @@ struct Work {
     int4 *tinfo;        // [ntiles] each tile's first site (x, y, z) and its counts: boundary pieces
                         // (bits 0-10), runs (bits 11-23), lattice of the launch (bits 24-29),
                         // TILE_ONE_PIECE (index fields)
-    int32_t *parent;    // [piece_cap] union-find parent over boundary pieces; tile t owns
-                        // the slice [t * MAX_BOUNDARY, t * MAX_BOUNDARY + piece count)
-    int32_t *key;       // [piece_cap] lattice-local site index of the piece's first site;
+    int32_t *parent;    // [ntiles * piece_stride] union-find parent over boundary pieces; tile t owns
+                        // the slice [t * piece_stride, t * piece_stride + piece count)
+    int32_t *key;       // [ntiles * piece_stride] lattice-local site index of the piece's first site;
                         // after piece_finalize: the label of the piece's cluster
-    int32_t *psize;     // [piece_cap] piece size; after piece_finalize: the cluster size at
+    int32_t *psize;     // [ntiles * piece_stride] piece size; after piece_finalize: the cluster size at
                         // the cluster's root piece, -1 elsewhere
     uint32_t *xcol;     // [ntiles * 2 * R/32] occupancy of each tile's first (x = 0) and last
                         // (x = lastX) column, one bit per tile row
@@ -85,12 +85,13 @@ struct Work {
     // interior, bit set where undetermined)
     uint32_t *neg, *pos;
     uint32_t *near_tile;   // [ntiles] whether the tile has near sites with a sign
-    int32_t *pvotes;    // [piece_cap]
+    int32_t *pvotes;    // [ntiles * piece_stride]
     uint32_t *tag;      // [ntiles * MAXRUNS / 16]
     int32_t *ovf;       // [ntiles] tiles with more runs than the fast tile pass holds
     int32_t *novf;      // [1] entries of ovf (reset by the occupancy pass of every call)
     int64_t piece_cap;  // bound of every global union-find loop: the entries of parent/key/psize
                         // (a path visits distinct pieces), or a lower test bound
+    int piece_stride;   // piece ids of a tile's slice (at least its boundary pieces, a multiple of 4)
     int32_t local_cap;  // bound of the shared-memory union retries: 0 = the tile's run count,
                         // > 0 a lower test bound
     // one slab of a lattice split along z (single-lattice launches only): added to every
@@ -228,8 +229,8 @@ __device__ __forceinline__ int top_bit(uint32_t w) {
 }
 // bits 0..x set
 __host__ __device__ __forceinline__ uint32_t le_mask(int x) { return (2u << x) - 1u; }
-// label of site x of a row (occupancy word m, run starts rs, first run id first): its run's
-// entry of lab, or -1 on the medium, where lab is not read -- before the row's first run there
+// label of site x of a row (occupancy word m, run starts rs, first run id first; le: bits 0..x):
+// its run's entry of lab, or -1 on the medium, where lab is not read -- before the row's first run there
 // is no entry that belongs to it, and before the tile's first none at all
 template <class Lab>
 __host__ __device__ __forceinline__ int site_label(uint32_t m, uint32_t rs, int first, uint32_t le, const Lab &lab) {

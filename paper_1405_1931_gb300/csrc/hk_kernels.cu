@@ -574,7 +574,7 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
         if (INDEX) __syncthreads();
 
         // the boundary pieces' records
-        const int base = (int)(t * SH::MAX_BOUNDARY);   // fixed slice of the piece table
+        const int base = (int)(t * W.piece_stride);     // fixed slice of the piece table
         const int nb_ = S.nbnd;
         if (FAST && nb_ > BL) {                 // block-uniform; nothing global written yet
             if (tid == 0) W.ovf[atomicAdd(W.novf, 1)] = (int32_t)t;
@@ -726,7 +726,7 @@ k_face_merge(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
     const int n1 = g.extYlo ? F[SH::OFF_CNT + 2] : 0;
     const int n2 = g.extZlo ? F[SH::OFF_CNT + 4] : 0;
     const int total = n0 + n1 + n2;
-    const int64_t base = t * SH::MAX_BOUNDARY;   // each tile owns a fixed slice of the piece table
+    const int64_t base = t * W.piece_stride;     // each tile owns a fixed slice of the piece table
     for (int i0 = 0; i0 < total; i0 += 32 * U) {
         int x[C], p[C];
 #pragma unroll
@@ -739,7 +739,7 @@ k_face_merge(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
                 const int hi = axis == 0 ? SH::OFF_HX : axis == 1 ? SH::OFF_HY : SH::OFF_HZ;
                 const int64_t nb = nbr[axis];
                 x[2 * u] = (int)(base + F[lo + j]);
-                x[2 * u + 1] = (int)(nb * SH::MAX_BOUNDARY + W.face[nb * SH::FACE_STRIDE + hi + j]);
+                x[2 * u + 1] = (int)(nb * W.piece_stride + W.face[nb * SH::FACE_STRIDE + hi + j]);
             } else {
                 x[2 * u] = x[2 * u + 1] = -1;   // no entry
             }
@@ -790,7 +790,7 @@ k_face_merge(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
 // --------------------------------------------------------------------------------------
 template <int NL, bool HOT>
 __global__ void __launch_bounds__(32 * PF_WARPS)
-k_piece_finalize(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles, int max_boundary) {
+k_piece_finalize(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
     grid_dep_wait();
     __shared__ int hot_target[PF_WARPS];   // per warp: the cluster root its pieces fed most, and the sum
     __shared__ int hot_sum[PF_WARPS], hot_votes[PF_WARPS];
@@ -805,7 +805,7 @@ k_piece_finalize(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles,
         for (int j0 = 0; j0 < nbnd; j0 += 32) {
             const int j = j0 + lane;
             const bool valid = j < nbnd;
-            const int pid = (int)t * max_boundary + j;
+            const int pid = (int)t * W.piece_stride + j;
             int root = -1, add = 0, vadd = 0;
             if (valid) {
                 root = g_find_ro(W.parent, pid, W.piece_cap, W.status);
@@ -1033,7 +1033,7 @@ struct FlatSmem {
     // (256 of them and five CTAs: 1.39 against 1.35 ms at 1024^3, p_c)
     static constexpr int GL = SH::MAX_BOUNDARY < 192 ? SH::MAX_BOUNDARY : 192;
     static constexpr int CC = SH::MR_FAST;                                       // staged run codes
-    static_assert(GL % 4 == 0 && CC % 8 == 0 && (SH::MAX_BOUNDARY * 4) % 16 == 0 && (SH::MAXRUNS * 2) % 16 == 0,
+    static_assert(GL % 4 == 0 && CC % 8 == 0 && SH::MAX_BOUNDARY % 4 == 0 && (SH::MAXRUNS * 2) % 16 == 0,
                   "bulk copies of whole 16-byte blocks from 16-byte aligned slices");
     // the staged tile (bulk copies)
     alignas(16) uint32_t words[SH::R];         // occupancy word of each row
@@ -1064,8 +1064,9 @@ k_flatten(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles, uint32
     grid_dep_wait();
     using SH = TileShape<TY, TZ>;
     using FS = FlatSmem<TY, TZ>;
-    constexpr int R = SH::R, NT = SH::NT, NW = NT / 32, MR = SH::MAXRUNS, MB = SH::MAX_BOUNDARY;
+    constexpr int R = SH::R, NT = SH::NT, NW = NT / 32, MR = SH::MAXRUNS;
     constexpr int GL = FS::GL, CC = FS::CC;
+    const int MB = W.piece_stride;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     FS &S = *reinterpret_cast<FS *>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -1103,7 +1104,7 @@ k_flatten(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles, uint32
         mbar_init(&S.bar, 1);
         fence_mbar_init();
         // the first tile's counts are not waited for: all that can be staged is copied
-        if (t < nt) issue(t, make_int4(0, 0, 0, GL | (CC << 11)));
+        if (t < nt) issue(t, make_int4(0, 0, 0, min(GL, MB) | (CC << 11)));
         uint32_t t1 = t, e1 = end;
         next_tile(t1, e1);
         if (t1 < nt) ti_next = W.tinfo[t1];
@@ -1357,8 +1358,9 @@ template <int TY, int TZ>
 __global__ void __launch_bounds__(TY * TZ) k_state(const LatDev L, Work W, int8_t *state, bool vec) {
     grid_dep_wait();
     using SH = TileShape<TY, TZ>;
-    constexpr int R = SH::R, NT = SH::NT, NW = NT / 32, MR = SH::MAXRUNS, MB = SH::MAX_BOUNDARY;
-    __shared__ int8_t ptag[MB];                        // tag of each boundary piece's cluster
+    constexpr int R = SH::R, NT = SH::NT, NW = NT / 32, MR = SH::MAXRUNS;
+    const int MB = W.piece_stride;
+    __shared__ int8_t ptag[SH::MAX_BOUNDARY];                        // tag of each boundary piece's cluster
     __shared__ uint2 row[R];                           // bits of the states 1 and -1 of each row
     __shared__ int warp_tmp[NW];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -1733,10 +1735,9 @@ static cudaError_t launch_all(const LatDev *lats, int n, const Plan &P, const Wo
     else if (ms.unions == 4) launch_dep(k_face_merge<TY, TZ, NL, 4>, gfm, 32 * FM_WARPS, 0, st, B, W, P.ntiles);
     else launch_dep(k_face_merge<TY, TZ, NL, 2>, gfm, 32 * FM_WARPS, 0, st, B, W, P.ntiles);
     mark(3);
-    constexpr int MB = SH::MAX_BOUNDARY;
     const unsigned gpf = (unsigned)((P.ntiles + PF_WARPS - 1) / PF_WARPS);
-    if (ms.hot) launch_dep(k_piece_finalize<NL, true>, gpf, 32 * PF_WARPS, 0, st, B, W, P.ntiles, MB);
-    else launch_dep(k_piece_finalize<NL, false>, gpf, 32 * PF_WARPS, 0, st, B, W, P.ntiles, MB);
+    if (ms.hot) launch_dep(k_piece_finalize<NL, true>, gpf, 32 * PF_WARPS, 0, st, B, W, P.ntiles);
+    else launch_dep(k_piece_finalize<NL, false>, gpf, 32 * PF_WARPS, 0, st, B, W, P.ntiles);
     mark(4);
     if constexpr (IX) {
         if (state) {                               // index fields: the state is all that is wanted

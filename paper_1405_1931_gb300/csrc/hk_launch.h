@@ -29,8 +29,38 @@ struct Plan {
     int64_t ntiles;      // tiles of all lattices in the launch
     int64_t nseg;        // row segments of all lattices
     int64_t nrows;       // lattice rows (y, z) of all lattices
-    int64_t piece_cap;   // ntiles * max_boundary
+    int64_t piece_cap;   // ntiles * piece_stride
+    int piece_stride;    // piece ids a tile owns, a multiple of 4 (16-byte blocks)
 };
+
+// Piece ids (tile * stride + k) are int32.
+constexpr int64_t MAX_PIECES = (int64_t)1 << 31;
+
+// Bound on the boundary pieces of a tile of one nx x ny x nz lattice.  Only an axis of several
+// tiles has faces with a neighbour; the pieces that touch a face are pairwise non-adjacent on
+// its grid, so at most half of its sites, rounded up, and a face is no larger than the lattice.
+inline int piece_bound(const TileInfo &ti, int nx, int ny, int nz) {
+    const int t[3] = {32, ti.ty, ti.tz}, n[3] = {nx, ny, nz};
+    int bound = 0;
+    for (int a = 0; a < 3; ++a) {
+        if (n[a] <= t[a]) continue;
+        const int b = (a + 1) % 3, c = (a + 2) % 3;
+        const int area = (n[b] < t[b] ? n[b] : t[b]) * (n[c] < t[c] ? n[c] : t[c]);
+        bound += (area + 1) / 2 * 2;
+    }
+    return bound > 4 ? (bound + 3) / 4 * 4 : 4;
+}
+
+// The slices of the piece table: the tile shape's own bound (max_boundary), which any lattice
+// may use, as long as the ids fit; a single lattice of more tiles than that (flat or thin
+// ones, whose tiles are mostly outside it: 32768 x 32768 x 1 has 2 M tiles) takes its own
+// bound.  False if the ids do not fit then either.
+inline bool plan_pieces(const TileInfo &ti, Plan &P, int nx, int ny, int nz) {
+    P.piece_stride = ti.max_boundary;
+    if (P.ntiles * P.piece_stride >= MAX_PIECES) P.piece_stride = piece_bound(ti, nx, ny, nz);
+    P.piece_cap = P.ntiles * P.piece_stride;
+    return P.piece_cap < MAX_PIECES;
+}
 
 constexpr int NUM_PASSES = 7;   // occupancy, tile_label, face_merge, piece_finalize, scan, lattice_finish, flatten
 
@@ -74,7 +104,7 @@ inline Layout make_layout(const TileInfo &ti, const Plan &P, bool votes = false)
 // two device int32 words (the STATUS_* flags, then the count of tiles handed to the
 // dense tile pass).  loop_cap > 0 lowers the bound of every capped union-find loop
 // (0: the natural bounds, the run count and the piece-table size).
-Work bind_work(char *base, const Layout &Ly, int32_t *status, int64_t piece_cap, int64_t loop_cap);
+Work bind_work(char *base, const Layout &Ly, int32_t *status, const Plan &P, int64_t loop_cap);
 
 bool tile_info(int ty, int tz, TileInfo &ti);
 

@@ -74,12 +74,12 @@ extern "C" int hk_label_noalloc(const float *phi, int nx, int ny, int nz, const 
 
     hk::TileInfo ti;
     hk::tile_info(TY, TZ, ti);
-    hk::Plan P{0, 0, 0, 0};
+    hk::Plan P{};
     const int64_t nbx = (nx + hk::TX - 1) / hk::TX, nby = (ny + TY - 1) / TY, nbz = (nz + TZ - 1) / TZ;
     P.ntiles = nbx * nby * nbz;
     P.nseg = nbx * (int64_t)ny * nz;
     P.nrows = (int64_t)ny * nz;
-    P.piece_cap = P.ntiles * ti.max_boundary;
+    if (!hk::plan_pieces(ti, P, nx, ny, nz)) return HK_ERR_TOO_LARGE;
     const hk::Layout Ly = hk::make_layout(ti, P);   // the same workspace layout as a context's
     if (HEADER_BYTES + Ly.total > SCRATCH_BYTES) return HK_ERR_TOO_LARGE;   // rejected before touching the GPU
 
@@ -93,7 +93,7 @@ extern "C" int hk_label_noalloc(const float *phi, int nx, int ny, int nz, const 
     // written earlier in the same call; the status word is cleared only when it is
     // read (here on the capacity path, or by hk_noalloc_sync_status), so a give-up is
     // reported even when several calls run before the check.
-    hk::Work W = hk::bind_work(base + HEADER_BYTES, Ly, reinterpret_cast<int32_t *>(base), P.piece_cap, 0);
+    hk::Work W = hk::bind_work(base + HEADER_BYTES, Ly, reinterpret_cast<int32_t *>(base), P, 0);
     W.neg = W.pos = W.near_tile = W.tag = nullptr;   // no interior/exterior identification here
     W.pvotes = nullptr;
 
