@@ -1479,14 +1479,17 @@ __global__ void __launch_bounds__(256) k_interior_update(const int8_t *prev, con
 
 // Dense form in place: a far site's state stays where it is, so only the 32-byte sectors of
 // states (32 sites, two lanes) that hold a near one are read and written, and away from
-// membranes the pass is the read of the index field: 729 capsules at 1024^3, 0.74 against
-// 0.98 ms with every state moved.  A warp half of whose sectors held one loads its next
-// states along with the index values, so that fields full of near sites lose little (0.32
-// against 0.30 ms for 343 M sites, a third of them near; 0.30 with a twentieth near).
-// Groups of four sites, read and written one by one, were faster on the capsules (0.71
-// ms) and slower on fuller fields (0.35 and 0.42 ms).  vec: both arrays 16-byte aligned.
-__global__ void __launch_bounds__(256, 8) k_interior_update_in_place(int8_t *state, const float *index, int64_t n,
-                                                                   bool vec) {
+// membranes the pass is the read of the index field.  A warp half of whose sectors held one
+// loads its next states along with the index values.  Bound by memory; four CTAs an SM draw
+// more from it than eight, above all on fields full of near sites, where eight lost to the
+// form that moves every state.  In us, with none / a twentieth / all of the sites near:
+//   2^30 sites   587 / 871 / 927 with four, 668 / 925 / 1013 with eight, 965 with every state moved
+//   343 M sites  191 / 284 / 294 with four, 214 / 295 / 323 with eight, 309 with every state moved
+// Groups of four sites, read and written one by one, were slower on fuller fields.
+// vec: both arrays 16-byte aligned.
+constexpr int UPDATE_IN_PLACE_CTAS = 4;   // of 256 threads, per SM
+__global__ void __launch_bounds__(256, UPDATE_IN_PLACE_CTAS)
+k_interior_update_in_place(int8_t *state, const float *index, int64_t n, bool vec) {
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
     int64_t done = 0;
     if (vec) {
@@ -1538,25 +1541,33 @@ __global__ void __launch_bounds__(256) k_interior_update_sites(int8_t *state, in
     }
 }
 
-static unsigned stream_grid(int64_t units) {
+static unsigned stream_grid(int64_t units, int per_sm = 8) {
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     int64_t g = (units + 255) / 256;
-    const int64_t cap = (int64_t)(nsm > 0 ? nsm : 1) * 8;
+    const int64_t cap = (int64_t)(nsm > 0 ? nsm : 1) * per_sm;
     if (g > cap) g = cap;
     return (unsigned)(g > 0 ? g : 1);
 }
 
-// In place, from this many sites on, only the states near a membrane are moved.  Below, both
-// arrays stay in L2 between steps and reading the states first is as fast or faster (12.3
-// against 14.4 us at 256^3); above, it is not (42.6 against 58.4 us at 400^3).
-constexpr int64_t UPDATE_IN_PLACE_MIN = (int64_t)1 << 25;
+// In place, only the states near a membrane are moved where the two arrays (5 bytes a site)
+// take more than four fifths of L2.  Below, both stay in L2 between steps and reading the
+// states along with the index is as fast or faster (84 MB: 12.3 us, against 12.3 to 14.3 from
+// none to all near; 105 MB: 17.6 against 14.4 to 17.9); above, it is not (115 MB: 19.5 against
+// 16.3 to 18.6; 168 MB: 26.7 against 22.5 to 25.5; L2 holds 135 MB).
+static bool update_in_place(int64_t n) {
+    int dev = 0, l2 = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
+    return 5 * n > (int64_t)l2 / 5 * 4;
+}
+
 cudaError_t launch_interior_update(const int8_t *prev, const float *index, int64_t n, int8_t *out, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    if (prev == out && n >= UPDATE_IN_PLACE_MIN) {
+    if (prev == out && update_in_place(n)) {
         const bool vec = ((reinterpret_cast<uintptr_t>(index) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
-        k_interior_update_in_place<<<stream_grid(vec ? n / 16 + 1 : n), 256, 0, st>>>(out, index, n, vec);
+        k_interior_update_in_place<<<stream_grid(vec ? n / 16 + 1 : n, UPDATE_IN_PLACE_CTAS), 256, 0, st>>>(out, index, n, vec);
         return cudaGetLastError();
     }
     const bool vec = ((reinterpret_cast<uintptr_t>(prev) | reinterpret_cast<uintptr_t>(index) |
