@@ -574,7 +574,7 @@ k_tile_label(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
         if (INDEX) __syncthreads();
 
         // the boundary pieces' records
-        const int base = (int)(t * W.piece_stride);     // fixed slice of the piece table
+        const int base = (int)t * W.piece_stride;       // fixed slice of the piece table (31-bit ids)
         const int nb_ = S.nbnd;
         if (FAST && nb_ > BL) {                 // block-uniform; nothing global written yet
             if (tid == 0) W.ovf[atomicAdd(W.novf, 1)] = (int32_t)t;
@@ -726,7 +726,7 @@ k_face_merge(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
     const int n1 = g.extYlo ? F[SH::OFF_CNT + 2] : 0;
     const int n2 = g.extZlo ? F[SH::OFF_CNT + 4] : 0;
     const int total = n0 + n1 + n2;
-    const int64_t base = t * W.piece_stride;     // each tile owns a fixed slice of the piece table
+    const int base = (int)t * W.piece_stride;    // each tile owns a fixed slice of the piece table (31-bit ids)
     for (int i0 = 0; i0 < total; i0 += 32 * U) {
         int x[C], p[C];
 #pragma unroll
@@ -738,8 +738,8 @@ k_face_merge(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles) {
                 const int lo = axis == 0 ? SH::OFF_LX : axis == 1 ? SH::OFF_LY : SH::OFF_LZ;
                 const int hi = axis == 0 ? SH::OFF_HX : axis == 1 ? SH::OFF_HY : SH::OFF_HZ;
                 const int64_t nb = nbr[axis];
-                x[2 * u] = (int)(base + F[lo + j]);
-                x[2 * u + 1] = (int)(nb * W.piece_stride + W.face[nb * SH::FACE_STRIDE + hi + j]);
+                x[2 * u] = base + F[lo + j];
+                x[2 * u + 1] = (int)nb * W.piece_stride + W.face[nb * SH::FACE_STRIDE + hi + j];
             } else {
                 x[2 * u] = x[2 * u + 1] = -1;   // no entry
             }
@@ -1066,7 +1066,7 @@ k_flatten(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles, uint32
     using FS = FlatSmem<TY, TZ>;
     constexpr int R = SH::R, NT = SH::NT, NW = NT / 32, MR = SH::MAXRUNS;
     constexpr int GL = FS::GL, CC = FS::CC;
-    const int MB = W.piece_stride;
+    const uint32_t MB = (uint32_t)W.piece_stride;      // t * MB is a piece id: 31 bits
     extern __shared__ __align__(128) unsigned char smem_raw[];
     FS &S = *reinterpret_cast<FS *>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -1085,8 +1085,8 @@ k_flatten(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles, uint32
         bulk_load(S.words, W.mask + (size_t)t * R, 4u * R, &S.bar);
         if (nc) bulk_load(S.codes, W.codes + (size_t)t * MR, 2u * nc, &S.bar);
         if (ng) {
-            bulk_load(S.tab, W.key + (size_t)t * MB, 4u * ng, &S.bar);
-            bulk_load(S.gsize, W.psize + (size_t)t * MB, 4u * ng, &S.bar);
+            bulk_load(S.tab, W.key + t * MB, 4u * ng, &S.bar);
+            bulk_load(S.gsize, W.psize + t * MB, 4u * ng, &S.bar);
         }
     };
     // CTA b takes the tiles [i span, (i + 1) span) of every item i = b, b + gridDim.x, ...
@@ -1104,7 +1104,7 @@ k_flatten(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles, uint32
         mbar_init(&S.bar, 1);
         fence_mbar_init();
         // the first tile's counts are not waited for: all that can be staged is copied
-        if (t < nt) issue(t, make_int4(0, 0, 0, min(GL, MB) | (CC << 11)));
+        if (t < nt) issue(t, make_int4(0, 0, 0, min(GL, (int)MB) | (CC << 11)));
         uint32_t t1 = t, e1 = end;
         next_tile(t1, e1);
         if (t1 < nt) ti_next = W.tinfo[t1];
@@ -1128,8 +1128,8 @@ k_flatten(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles, uint32
                 S.words[tid] = W.mask[(size_t)t * R + tid];
                 for (int k = tid; k < total && k < CC; k += NT) S.codes[k] = W.codes[(size_t)t * MR + k];
                 for (int k = tid; k < nb && k < GL; k += NT) {
-                    S.tab[k] = W.key[(size_t)t * MB + k];
-                    S.gsize[k] = W.psize[(size_t)t * MB + k];
+                    S.tab[k] = W.key[t * MB + k];
+                    S.gsize[k] = W.psize[t * MB + k];
                 }
             }
             m = S.words[tid];
@@ -1193,7 +1193,6 @@ k_flatten(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles, uint32
 
         // The next two steps are compiled for tiles that are staged whole and for others.
         const uint16_t *C = W.codes + (size_t)t * MR;
-        const int32_t *gl_g = W.key + (size_t)t * MB, *gs_g = W.psize + (size_t)t * MB;
         auto decode_runs = [&](auto BIG) {
             constexpr bool big = decltype(BIG)::value;
             // one run per thread: the label of its boundary piece's cluster, or of the first
@@ -1208,8 +1207,8 @@ k_flatten(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles, uint32
                 const bool isb = (c & CODE_BOUNDARY) != 0;
                 int lab, gs;
                 if (big && isb && k >= GL) {
-                    lab = __ldg(gl_g + k);
-                    gs = __ldg(gs_g + k);
+                    lab = __ldg(W.key + (t * MB + k));
+                    gs = __ldg(W.psize + (t * MB + k));
                 } else {
                     lab = S.tab[isb ? k : GL + (k >> 5)];
                     gs = S.gsize[isb ? k : GL];
@@ -1242,7 +1241,7 @@ k_flatten(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles, uint32
                 const int id = rb + __ffs(w) - 1;
                 const int c = id < CC ? (int)S.codes[id] : (int)__ldg(C + id);
                 const uint32_t *T = W.tag + (size_t)t * (MR / 16) + 2 * (id >> 5);
-                const int v = (c & CODE_BOUNDARY) ? W.pvotes[(size_t)t * MB + (c & CODE_LOW)]
+                const int v = (c & CODE_BOUNDARY) ? W.pvotes[t * MB + (c & CODE_LOW)]
                             : (T[0] >> (id & 31)) & 1u ? -1 : (T[1] >> (id & 31)) & 1u ? 0 : 1;
                 L.inside[k] = (int8_t)(v < 0 ? 1 : (v > 0 ? 0 : -1));
             }
@@ -1274,7 +1273,7 @@ k_flatten(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles, uint32
                     const int c = (!bigt || id < CC) ? (int)S.codes[id] : (int)__ldg(C + id);
                     const int k = c & CODE_LOW;
                     const bool isb = (c & CODE_BOUNDARY) != 0;
-                    const int gs = (bigt && isb && k >= GL) ? __ldg(gs_g + k) : S.gsize[isb ? k : GL];
+                    const int gs = (bigt && isb && k >= GL) ? __ldg(W.psize + (t * MB + k)) : S.gsize[isb ? k : GL];
                     const int size = isb ? gs : k;
                     if (SLAB && rank < cap) W.roots[rank] = S.lab[id];   // a root's label is its own first site
                     S.pend[r][(rank + place) & 7u] = size;
@@ -1359,16 +1358,16 @@ __global__ void __launch_bounds__(TY * TZ) k_state(const LatDev L, Work W, int8_
     grid_dep_wait();
     using SH = TileShape<TY, TZ>;
     constexpr int R = SH::R, NT = SH::NT, NW = NT / 32, MR = SH::MAXRUNS;
-    const int MB = W.piece_stride;
-    __shared__ int8_t ptag[SH::MAX_BOUNDARY];                        // tag of each boundary piece's cluster
+    __shared__ int8_t ptag[SH::MAX_BOUNDARY];          // tag of each boundary piece's cluster
     __shared__ uint2 row[R];                           // bits of the states 1 and -1 of each row
     __shared__ int warp_tmp[NW];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int64_t t = blockIdx.x;
+    const int32_t *parent = W.parent + blockIdx.x * (uint32_t)W.piece_stride;   // a piece id: 31 bits
     const int4 ti = W.tinfo[t];
     const int nb = ti.w & 0x7ff;
     const uint32_t m = W.mask[t * R + tid], near_in = W.neg[t * R + tid];
-    const int root0 = W.parent[t * MB];                // of piece 0, if there is one
+    const int root0 = parent[0];                       // of piece 0, if there is one
     const uint32_t rs = run_starts(m);
     uint32_t ones = near_in, ties = 0;
     if (ti.w & TILE_ONE_PIECE) {                       // uniform: the tile's far sites are one piece
@@ -1384,7 +1383,7 @@ __global__ void __launch_bounds__(TY * TZ) k_state(const LatDev L, Work W, int8_
         }
         if (lane == 31) warp_tmp[wid] = inc;
         for (int k = tid; k < nb; k += NT) {
-            const int v = W.pvotes[W.parent[t * MB + k]];  // piece_finalize left every piece at its root
+            const int v = W.pvotes[parent[k]];             // piece_finalize left every piece at its root
             ptag[k] = (int8_t)(v < 0 ? 1 : (v > 0 ? 0 : -1));
         }
         __syncthreads();
