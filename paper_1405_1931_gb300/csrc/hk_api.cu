@@ -309,13 +309,12 @@ int run_lattices(hk_ctx *ctx, const hk_lattice *lats, int n, cudaStream_t st, bo
             all_cluster = all_cluster && hk::cluster_fits(lats[i].nx, lats[i].ny, lats[i].nz);
         }
         if (all_one || all_cluster) {
-            // The smallest lattices finish sooner on one CTA (a call of one: 14.4 against 15.4 us at
-            // 8^3; at 16^3 17.3 against 18.5 us for p = 0.3 but 20.5 against 18.5 for p = 0.45).
-            // Above that clusters win while they fill about half of the device's cluster slots, past
+            // The smallest lattices finish sooner on one CTA (hk::one_cta_wins).  Above that
+            // clusters win while they fill about half of the device's cluster slots, past
             // which lattices that fit one CTA each take one (at 32^3 with 7 slots of 16 CTAs: 1 lattice
             // 20.6 against 26.6 us, 4 lattices 24.6 against 28.7, 8 lattices 46.7 against 28.3).
             bool tiny = all_one;
-            for (int i = 0; i < n && tiny; ++i) tiny = (int64_t)lats[i].nx * lats[i].ny * lats[i].nz <= 2048;
+            for (int i = 0; i < n && tiny; ++i) tiny = hk::one_cta_wins(lats[i].nx, lats[i].ny, lats[i].nz);
             const bool cluster = all_cluster && (!all_one || (!tiny && 2 * n <= hk::cluster_slots() + 1));
             int rc_cap = HK_OK;
             for (int c0 = 0; c0 < n; c0 += hk::MAX_LAT_PER_LAUNCH) {

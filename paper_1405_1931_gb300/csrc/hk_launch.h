@@ -115,6 +115,15 @@ constexpr int SMALL_MAX_SITES = 32768;
 constexpr int SMALL_MAX_SEG = 2048;
 constexpr int SMALL_MAX_RUNS = 16384 + 2048;
 bool small_fits(int nx, int ny, int nz);
+// A lattice that one CTA labels sooner than a cluster does, whatever its field: at most 128
+// rows of at most 12 sites, or a single row of at most 2048.  One CTA gives a row to a
+// thread, so long rows of many runs and many rows both make it the slower one.  Means over
+// fourteen fields, one CTA / cluster: 8^3 14.5 / 15.6 us, 10^3 15.3 / 17.8, 12 x 8 x 16
+// 15.6 / 16.0, 2048 x 1 x 1 10.6 / 15.0; beyond the line single fields lose: 32 x 8 x 8 at p =
+// 0.45 26.7 / 18.9, 1 x 32 x 64 full 39.4 / 18.5, 1 x 1 x 2048 full 33 / 20.
+inline bool one_cta_wins(int nx, int ny, int nz) {
+    return (nx <= 12 && (int64_t)ny * nz <= 128) || (nx <= 2048 && ny == 1 && nz == 1);
+}
 // The cluster form (hk_small.cu): a cluster of CS CTAs on CS SMs labels one lattice
 // whose rows, split into CS equal blocks, come to at most 1024 row segments a block.
 // CS is 16 where the device co-schedules a cluster that large, else 8 (64^3 fits
