@@ -62,6 +62,19 @@ struct FastDiv {
     __device__ __forceinline__ uint32_t operator()(uint32_t x) const { return (uint32_t)((x * m) >> 32); }
 };
 
+// Links make chains: of stripes across x a run hangs on the row below it, that one on the
+// next, as many as there are rows.  From CHAIN links on each run is first pointed at what its
+// parent points at, once a halving of the longest possible chain (an ancestor, so it does not
+// matter which of two such stores a read meets).
+constexpr int CHAIN = 24;
+template <int NT>
+__device__ __forceinline__ void shorten_chains(int *par, int total, int longest) {
+    for (; longest > CHAIN; longest >>= 1) {
+        for (int i = threadIdx.x; i < total; i += NT) par[i] = par[par[i]];
+        __syncthreads();
+    }
+}
+
 // the run of segment s (first run id b, occupancy word w) holding bit x
 __device__ __forceinline__ int srun(int b, uint32_t w, int x) { return b + __popc(run_starts(w) & le_mask(x)) - 1; }
 
@@ -187,32 +200,48 @@ __global__ void __launch_bounds__(SNT, 1) k_small_label(const __grid_constant__ 
         }
     }
     __syncthreads();
+    shorten_chains<SNT>(S.par, total, min(ny + nz, total));
     const int cap = (local_cap > 0 && local_cap < total) ? local_cap : total;
+    // (each kind of pair has one loop around one union: the kernel runs once through its code,
+    // and fetching that counts: 17.4 us for 8 lattices of 16^3, 18.0 with two loops for each)
     const int lastbit = (nx - 1) & 31;   // bit of x = nx - 1 in the last segment of a row
     for (int h = 0; h < 2; ++h) {
         const int s = tid + h * SNT;
         const uint32_t w = h ? w_b : w_a;
         if (s >= nseg || !w) continue;
         const int b = first_run(h);
-        const int q = (int)div_nbx((uint32_t)s), bx = s - q * nbx, z = (int)div_ny((uint32_t)q), y = q - z * ny;
-        auto join = [&](int t, uint32_t os) {   // the pairs of segments s and t that start at bits os
+#pragma unroll 1
+        for (int d = 0; d < 2; ++d) {                // the pairs with the lower rows along z and y
+            uint32_t os = d ? rest_y[h] : rest_z[h];
+            if (!os) continue;
+            const int t = d ? s - nbx : s - nbx * ny, bt = S.sb[t];
             const uint32_t wt = S.m[t];
-            const int bt = S.sb[t];
-            while (os) {
+            for (; os; os &= os - 1u) {
                 const int x = top_bit(os & (0u - os));
-                os &= os - 1;
                 s_union(S.par, srun(b, w, x), srun(bt, wt, x), cap, status);
             }
-        };
-        if (rest_z[h]) join(s - nbx * ny, rest_z[h]);
-        if (rest_y[h]) join(s - nbx, rest_y[h]);
-        if (y == 0 && L.per[1] && ny >= 2) join(s + (ny - 1) * nbx, run_starts(w & S.m[s + (ny - 1) * nbx]));
-        if (z == 0 && L.per[2] && nz >= 2) join(s + (nz - 1) * nbx * ny, run_starts(w & S.m[s + (nz - 1) * nbx * ny]));
-        if ((w & 1u) && bx > 0 && (S.m[s - 1] >> 31))
-            s_union(S.par, b, srun(S.sb[s - 1], S.m[s - 1], 31), cap, status);
-        if ((w & 1u) && bx == 0 && L.per[0] && nx >= 2) {
-            const int t = s + nbx - 1;
-            if ((S.m[t] >> lastbit) & 1u) s_union(S.par, b, srun(S.sb[t], S.m[t], lastbit), cap, status);
+        }
+        if (w & 1u) {                                // along x: the segment before, or the periodic edge
+            const int bx = s - (int)div_nbx((uint32_t)s) * nbx, t = bx > 0 ? s - 1 : s + nbx - 1, x = bx > 0 ? 31 : lastbit;
+            if ((bx > 0 || (L.per[0] && nx >= 2)) && ((S.m[t] >> x) & 1u))
+                s_union(S.par, b, srun(S.sb[t], S.m[t], x), cap, status);
+        }
+    }
+    // The periodic edges along y and z.  A find from the far side climbs a row's links, one
+    // for every row of stripes across x, so the pairs of a segment are shared out by nibbles
+    // over the warps.
+    {
+        const int wrap_y = L.per[1] && ny >= 2 ? nbx * nz : 0, wraps = wrap_y + (L.per[2] && nz >= 2 ? nbx * ny : 0);
+        const int shares = nx > 16 ? 3 : nx > 8 ? 2 : nx > 4 ? 1 : 0;   // log2; a word has pairs at its first nx bits only
+        const uint32_t part = shares ? 0xfu << (4 * (wid & ((1 << shares) - 1))) : ~0u;
+        for (int j = (wid >> shares) * 32 + lane; j < wraps; j += (NW >> shares) * 32) {
+            const int z = (int)div_nbx((uint32_t)j), s = j < wrap_y ? z * ny * nbx + j - z * nbx : j - wrap_y;
+            const int t = s + (j < wrap_y ? (ny - 1) * nbx : (nz - 1) * nbx * ny), b = S.sb[s], bt = S.sb[t];
+            const uint32_t w = S.m[s], wt = S.m[t];
+            for (uint32_t os = run_starts(w & wt) & part; os; os &= os - 1u) {
+                const int x = top_bit(os & (0u - os));
+                s_union(S.par, srun(b, w, x), srun(bt, wt, x), cap, status);
+            }
         }
     }
     __syncthreads();
@@ -532,14 +561,22 @@ __global__ void __cluster_dims__(1 << CSB, 1, 1) __launch_bounds__(CNT, 1)
         // the edges inside the CTA, one segment a thread: as in the tile pass a run's first
         // pair with a lower row is a store into its own node and a z pair whose site is
         // joined through its y neighbours is left out; the others follow after a
-        // barrier, eight shares a segment (a byte of its z or y pairs and some of its edges)
-        // over as many threads as there are
+        // barrier, and with them those of the periodic edges along y and z (a segment has
+        // those in place of its pairs with a lower row): 16 shares a segment (a nibble of its
+        // z or y pairs) over as many threads as there are, since a find may climb a chain of
+        // links as long as the lattice is wide (stripes across x)
         // (from half as many segments as threads on: all listed by a scan and taken in turn,
         // 51 against 54 us at 64 x 96 x 80, p_c)
         const int row = nbx * ny;
         uint32_t osy = 0, osz = 0;
+        auto below = [&](int ls, bool z_) {          // the segment of ls's y or z pairs
+            const int q = (int)div_nbx((uint32_t)(seg0 + ls)), z = (int)div_ny((uint32_t)q);
+            if (z_) return z > 0 ? ls - row : ls + (nz - 1) * row;
+            return q > z * ny ? ls - nbx : ls + (ny - 1) * nbx;
+        };
         if (tid < nseg) {
             const int ls = tid, q = (int)div_nbx((uint32_t)(seg0 + ls)), z = (int)div_ny((uint32_t)q), y = q - z * ny;
+            const int wy = ls + (ny - 1) * nbx, wz = ls + (nz - 1) * row;
             const uint32_t w = S.m[ls];
             const uint32_t my = y > 0 && ls >= nbx ? S.m[ls - nbx] : 0u, mz = z > 0 && ls >= row ? S.m[ls - row] : 0u;
             const uint32_t oy = w & my, oz = w & mz, uy = fill_up(w, oy), rs = run_starts(w);
@@ -558,6 +595,13 @@ __global__ void __cluster_dims__(1 << CSB, 1, 1) __launch_bounds__(CNT, 1)
                 const bool iy = (my & low) != 0u;
                 S.par[b + __popc(rs & le) - 1] = (iy ? by : bz) + __popc((iy ? rsy : rsz) & le) - 1;
             }
+            if (y == 0 && L.per[1] && ny >= 2 && wy < nseg) osy = run_starts(w & S.m[wy]);
+            if (z == 0 && L.per[2] && nz >= 2 && wz < nseg) osz = run_starts(w & S.m[wz]);
+        }
+        const int longest = min(ny, rp) + rp / ny;   // links of a chain: y goes down, then z
+        if (longest > CHAIN) {
+            __syncthreads();
+            shorten_chains<CNT>(S.par, total, min(longest, total));
         }
         bool listed = false;                         // CTA-uniform
         if (2 * nseg >= CNT) {
@@ -566,7 +610,6 @@ __global__ void __cluster_dims__(1 << CSB, 1, 1) __launch_bounds__(CNT, 1)
             listed = npairs <= CRUN;
             if (listed) {
                 auto list = [&](int t, uint32_t os) {
-                    if (!os) return;
                     const uint32_t w = S.m[tid], wt = S.m[t];
                     const int b = S.sb[tid], bt = S.sb[t];
                     for (; os; os &= os - 1u) {
@@ -574,50 +617,38 @@ __global__ void __cluster_dims__(1 << CSB, 1, 1) __launch_bounds__(CNT, 1)
                         S.sz[j++] = (srun(b, w, x) << CRUN_BITS) | srun(bt, wt, x);
                     }
                 };
-                list(tid - row, osz);
-                list(tid - nbx, osy);
+                if (osz) list(below(tid, true), osz);
+                if (osy) list(below(tid, false), osy);
                 __syncthreads();
                 for (int k = tid; k < npairs; k += CNT)
                     s_union(S.par, S.sz[k] >> CRUN_BITS, S.sz[k] & (CRUN - 1), lcap, status);
             }
         }
-        if (!listed && tid < nseg) {
-            S.sz[tid] = (int)osz;
-            S.sz[CSEG + tid] = (int)osy;
+        if (!listed) {
+            if (tid < nseg) {
+                S.sz[tid] = (int)osz;
+                S.sz[CSEG + tid] = (int)osy;
+            }
+            __syncthreads();
         }
-        __syncthreads();
         const int groups = nseg > 0 ? CNT / nseg : 1, group = nseg > 0 ? tid / nseg : CNT;
-        for (int share = (listed ? 4 : 0) + group; group < groups && share < 8; share += groups) {
+        for (int share = (listed ? 16 : 0) + group; group < groups && share < 17; share += groups) {
             const int ls = tid - group * nseg;
             const uint32_t w = S.m[ls];
-            if (!w) continue;
-            const int b = S.sb[ls];
-            auto join = [&](int t, uint32_t os) {   // the pairs of segments ls and t that start at bits os
-                if (!os) return;
+            if (share < 16) {
+                uint32_t os = (uint32_t)S.sz[share < 8 ? ls : CSEG + ls] & (0xfu << (4 * (share & 7)));
+                if (!os) continue;
+                const int t = below(ls, share < 8), b = S.sb[ls], bt = S.sb[t];
                 const uint32_t wt = S.m[t];
-                const int bt = S.sb[t];
                 for (; os; os &= os - 1u) {
                     const int x = top_bit(os & (0u - os));
                     s_union(S.par, srun(b, w, x), srun(bt, wt, x), lcap, status);
                 }
-            };
-            const uint32_t part = 0xffu << (8 * (share & 3));
-            if (!listed) {
-                if (share < 4) join(ls - row, (uint32_t)S.sz[ls] & part);
-                else join(ls - nbx, (uint32_t)S.sz[CSEG + ls] & part);
-            }
-            if (share >= 4 && share < 7) {           // periodic edges and rows of several segments
-                const int q = (int)div_nbx((uint32_t)(seg0 + ls)), bx = seg0 + ls - q * nbx, z = (int)div_ny((uint32_t)q);
-                const int y = q - z * ny, wy = ls + (ny - 1) * nbx, wz = ls + (nz - 1) * row;
-                if (share == 4 && y == 0 && L.per[1] && ny >= 2 && wy < nseg) join(wy, run_starts(w & S.m[wy]));
-                if (share == 5 && z == 0 && L.per[2] && nz >= 2 && wz < nseg) join(wz, run_starts(w & S.m[wz]));
-                if (share == 6 && (w & 1u)) {
-                    if (bx > 0 && (S.m[ls - 1] >> 31)) s_union(S.par, b, srun(S.sb[ls - 1], S.m[ls - 1], 31), lcap, status);
-                    if (bx == 0 && L.per[0] && nx >= 2) {
-                        const int t = ls + nbx - 1;
-                        if ((S.m[t] >> lastbit) & 1u) s_union(S.par, b, srun(S.sb[t], S.m[t], lastbit), lcap, status);
-                    }
-                }
+            } else if (w & 1u) {                     // along x: rows of several segments, the periodic edge
+                const int bx = seg0 + ls - (int)div_nbx((uint32_t)(seg0 + ls)) * nbx;
+                const int t = bx > 0 ? ls - 1 : ls + nbx - 1, x = bx > 0 ? 31 : lastbit;
+                if ((bx > 0 || (L.per[0] && nx >= 2)) && ((S.m[t] >> x) & 1u))
+                    s_union(S.par, S.sb[ls], srun(S.sb[t], S.m[t], x), lcap, status);
             }
         }
         __syncthreads();
