@@ -27,6 +27,7 @@
 #include <cstdint>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "hk_device.cuh"
 #include "hk_launch.h"
@@ -128,24 +129,28 @@ __global__ void __launch_bounds__(SNT, 1) k_small_label(const __grid_constant__ 
     // a1: occupancy words; each warp keeps up to 32 segments' loads in flight (a 32^3
     // lattice in one round trip)
     constexpr int INF = 32;
-    for (int s0 = wid; s0 < nseg; s0 += NW * INF) {
-        float v[INF];
+    auto read_words = [&](auto FLAT) {
+        for (int s0 = wid; s0 < nseg; s0 += NW * INF) {
+            float v[INF];
 #pragma unroll
-        for (int j = 0; j < INF; ++j) {
-            const int s = s0 + NW * j;
-            if (flat) {
-                v[j] = s < nseg ? __ldg(L.phi + 32 * s + lane) : 0.0f;
-            } else {
-                const int q = (int)div_nbx((uint32_t)s), x = (s - q * nbx) * 32 + lane;
-                v[j] = (s < nseg && x < nx) ? __ldg(L.phi + (int64_t)q * nx + x) : 0.0f;
+            for (int j = 0; j < INF; ++j) {
+                const int s = s0 + NW * j;
+                if (decltype(FLAT)::value) {
+                    v[j] = s < nseg ? __ldg(L.phi + 32 * s + lane) : 0.0f;
+                } else {
+                    const int q = (int)div_nbx((uint32_t)s), x = (s - q * nbx) * 32 + lane;
+                    v[j] = (s < nseg && x < nx) ? __ldg(L.phi + (int64_t)q * nx + x) : 0.0f;
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < INF; ++j) {
+                const uint32_t w = __ballot_sync(0xffffffffu, occupied(v[j], L.occ_mode));
+                if (lane == 0 && s0 + NW * j < nseg) S.m[s0 + NW * j] = w;
             }
         }
-#pragma unroll
-        for (int j = 0; j < INF; ++j) {
-            const uint32_t w = __ballot_sync(0xffffffffu, occupied(v[j], L.occ_mode));
-            if (lane == 0 && s0 + NW * j < nseg) S.m[s0 + NW * j] = w;
-        }
-    }
+    };
+    if (flat) read_words(std::true_type{});
+    else read_words(std::false_type{});
     __syncthreads();
 
     // a2: run ids: one scan of the run counts of segments t (low half) and t + SNT
@@ -284,17 +289,21 @@ __global__ void __launch_bounds__(SNT, 1) k_small_label(const __grid_constant__ 
     __syncthreads();
 
     // a5: labels, one warp per segment, one lane per site
+    auto write_labels = [&](auto FLAT) {
 #pragma unroll 4
-    for (int s = wid; s < nseg; s += NW) {
-        const uint32_t w = S.m[s];
-        const int lab = ((w >> lane) & 1u) ? S.sz[S.par[srun(S.sb[s], w, lane)]] : -1;
-        if (flat) {
-            L.labels[32 * s + lane] = lab;
-        } else {
-            const int q = (int)div_nbx((uint32_t)s), x = (s - q * nbx) * 32 + lane;
-            if (x < nx) L.labels[(int64_t)q * nx + x] = lab;
+        for (int s = wid; s < nseg; s += NW) {
+            const uint32_t w = S.m[s];
+            const int lab = ((w >> lane) & 1u) ? S.sz[S.par[srun(S.sb[s], w, lane)]] : -1;
+            if (decltype(FLAT)::value) {
+                L.labels[32 * s + lane] = lab;
+            } else {
+                const int q = (int)div_nbx((uint32_t)s), x = (s - q * nbx) * 32 + lane;
+                if (x < nx) L.labels[(int64_t)q * nx + x] = lab;
+            }
         }
-    }
+    };
+    if (flat) write_labels(std::true_type{});
+    else write_labels(std::false_type{});
     __syncthreads();
     if (tid < 32 && L.hist) L.hist[tid] = S.hist[tid];
     if (tid == 0 && L.ncl) L.ncl[0] = nclus;
