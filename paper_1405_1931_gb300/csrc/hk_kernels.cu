@@ -1113,7 +1113,8 @@ k_flatten(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles, uint32
     bool prefetch = true;
     uint32_t parity = 0;
     int cur_lat = -1;
-    uint32_t rank = 0, lo = 0;                         // of this row: next rank, first one not written
+    constexpr uint32_t NO_RANK = ~0u;                  // ranks stay below 2^30
+    uint32_t rank = NO_RANK, lo = NO_RANK;             // of this row: next rank, first one not written
     while (t < nt) {
         uint32_t m, rs;
         int inc;
@@ -1156,10 +1157,13 @@ k_flatten(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles, uint32
         if (tid == 0 && L.ncl && (ti.x | ti.y | ti.z) == 0)
             L.ncl[0] = (int64_t)(uint32_t)(W.pre[L.row0 + (int64_t)L.nz * L.ny] - W.pre[L.row0]);
         // Rank base of this row: the roots of the lattice's earlier rows, then of this row's
-        // earlier segments; carried on while the tiles follow each other along x.
+        // earlier segments; carried on while the tiles follow each other along x.  Looked up
+        // in the first tile where one of the warp's rows has a run (looked up whether there is one
+        // or not, an empty 65536 x 64 x 4 took 589 us against 282).
         const int q = (ti.z + lz) * L.ny + (ti.y + ly);
         const bool valid_row = ti.y + ly < L.ny && ti.z + lz < L.nz;
-        if ((fresh || ti.x == 0) && valid_row) {
+        if (fresh || ti.x == 0) rank = lo = NO_RANK;
+        if (__any_sync(0xffffffffu, rs != 0u) && rank == NO_RANK && valid_row) {
             rank = W.pre[L.row0 + q] - W.pre[L.row0];
             if (ti.x) rank += bytes_sum(W.cnt, L.seg0 + (int64_t)q * L.nbx, ti.x / TX);
             lo = rank;
