@@ -338,13 +338,12 @@ __device__ __forceinline__ void s_union(int *par, int a, int b, int cap, int32_t
     atomicOr(status, STATUS_LOCAL_LOOP);
 }
 
-// join the runs of row r and row q that overlap along x (used for the rare in-tile wraps)
-__device__ __forceinline__ void join_rows(int *par, uint32_t m, int rb, uint32_t mq, int rbq, int cap,
+// join the runs of row r and row q that overlap along x (used for the rare in-tile wraps), for
+// the overlaps that start at bits of part
+__device__ __forceinline__ void join_rows(int *par, uint32_t m, int rb, uint32_t mq, int rbq, uint32_t part, int cap,
                                           int32_t *status) {
-    uint32_t o = m & mq;
-    if (!o) return;
     const uint32_t rs = run_starts(m), rsq = run_starts(mq);
-    uint32_t os = run_starts(o);
+    uint32_t os = run_starts(m & mq) & part;
     while (os) {
         int x = __ffs(os) - 1;
         os &= os - 1;
