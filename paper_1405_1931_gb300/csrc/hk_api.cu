@@ -312,7 +312,7 @@ int run_lattices(hk_ctx *ctx, const hk_lattice *lats, int n, cudaStream_t st, bo
             // The smallest lattices finish sooner on one CTA (hk::one_cta_wins).  Above that
             // clusters win while they fill about half of the device's cluster slots, past
             // which lattices that fit one CTA each take one (at 32^3 with 7 slots of 16 CTAs: 1 lattice
-            // 20.6 against 26.6 us, 4 lattices 24.6 against 28.7, 8 lattices 46.7 against 28.3).
+            // 20.5 against 24.1 us, 4 lattices 22.0 against 24.6, 8 lattices 38.9 against 24.6).
             bool tiny = all_one;
             for (int i = 0; i < n && tiny; ++i) tiny = hk::one_cta_wins(lats[i].nx, lats[i].ny, lats[i].nz);
             const bool cluster = all_cluster && (!all_one || (!tiny && 2 * n <= hk::cluster_slots() + 1));

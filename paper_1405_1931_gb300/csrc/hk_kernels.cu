@@ -240,10 +240,10 @@ __global__ void __launch_bounds__(256) k_occupancy_tma(const __grid_constant__ T
 // --------------------------------------------------------------------------------------
 // K1: tile labelling from the occupancy words (one tile per CTA)
 //
-// Bound by instruction issue (90 % of its rate): 2 warp instructions a site at p_c.  With
+// Bound by instruction issue (90 % of its rate at 512^3): 2 warp instructions a site at p_c.  With
 // most pairs linked or left out instead of united, and with boundary pieces listed by the
-// run that first touches a face instead of in passes over all runs: 1.90 against 2.38 ms
-// at 1024^3, p_c, 0.80 against 1.06 ms on blocks of 16^3, 0.127 against 0.148 ms on a
+// run that first touches a face instead of in passes over all runs: 1.82 against 2.38 ms
+// at 1024^3, p_c, 0.79 against 1.06 ms on blocks of 16^3, 0.125 against 0.148 ms on a
 // 512^3 bijel.
 // --------------------------------------------------------------------------------------
 template <int TY, int TZ, int CAP, int BL, bool INDEX>
@@ -1022,11 +1022,15 @@ __global__ void __launch_bounds__(SCAN_NT) k_scan_apply(const __grid_constant__ 
 // global memory.  The next tile's record, words, codes and boundary pieces come by bulk
 // copy while the labels are written.
 //
-// Bound by instruction issue at p_c (1.2 warp instructions a site, 70 % of the issue
-// rate) and by the label stores on fields of long runs.  Against a loop over each row's
-// runs that decoded, ranked and filled them into a staged tile for a TMA store: 1.33
-// against 1.57 ms at 1024^3, p_c, 0.88 against 0.92 ms on blocks of 16^3, 0.105 against
-// 0.126 ms on a 512^3 bijel, 52 against 65 us at 387 x 283 x 221 (unaligned rows).
+// Bound by instruction issue at p_c (1.2 warp instructions a site, 72 % of the issue
+// rate at 512^3); on fields of long runs the label stores are two thirds of it.  Against
+// a loop over each row's runs that decoded, ranked and filled them into a staged tile for a
+// TMA store: 1.35 against 1.57 ms at 1024^3, p_c, 0.109 against 0.126 ms on a 512^3 bijel, 53
+// against 65 us at 387 x 283 x 221 (unaligned rows), and no faster on blocks of 16^3 (0.91
+// against 0.92 ms).  Slower on sixteen runs a row (stripes of one site at 512^3: 0.31 against
+// 0.19 ms, of a call of 1.14 against 1.46), whose codes do not fit the staged ones, and on
+// rows of four sites (0.13 against 0.09 ms at 4 x 2048 x 2048, p_c), where an eighth of the
+// lanes store.
 // --------------------------------------------------------------------------------------
 // Resident threads of an SM (40 registers each).  2048 (32 registers, spills): 1.63 ms at
 // 1024^3, p_c, against 1.50 for 1536 and 1.59 for 1280, in the form of that time.
@@ -1363,9 +1367,10 @@ k_flatten(const __grid_constant__ LatBatch<NL> B, Work W, int64_t ntiles, uint32
 // site the side its value names (step 2: -d inside, +d outside), 1 for I < 0 and 0
 // otherwise.  Like flatten it decodes the runs of each tile, but it needs neither ranks
 // nor labels: it reads the words and codes and writes a byte a site.  One tile per CTA,
-// one row per thread; a tile of one piece, as most are, needs no codes.  Bound by the
-// latency of its few loads: 729 capsules at 1024^3 take 0.30 ms, a fifth of the copy
-// rate for its 1.3 GB (0.51 with codes read in every tile and half sectors stored).
+// one row per thread; a tile of one piece, as most are, needs no codes.  729 capsules at
+// 1024^3 take 0.30 ms, two thirds of the copy rate for its 1.3 GB (0.51 with codes read in
+// every tile and half sectors stored); the rest is the chain of dependent loads at a CTA's
+// start (record, root, votes), which a 64-bit product in the root's address made 7 % longer.
 // --------------------------------------------------------------------------------------
 template <int TY, int TZ>
 __global__ void __launch_bounds__(TY * TZ) k_state(const LatDev L, Work W, int8_t *state, bool vec) {

@@ -1,7 +1,7 @@
 // hk_small.cu -- one launch for small lattices: one CTA labels a whole lattice of at
 // most SMALL_MAX_SITES sites in shared memory (a batch of such lattices: one CTA each).
 //
-// The tiled passes of hk_kernels.cu need about ten launches per call, whose gaps are
+// The tiled passes of hk_kernels.cu need eight launches per call, whose gaps are
 // the whole cost of a 32^3 lattice.  Here every step runs in one kernel, separated by
 // barriers instead of launches:
 //   a1  occupancy phi > 0 (Sec. 2) as one 32-bit word per row segment (32 sites along x);
@@ -17,10 +17,10 @@
 // (its smallest run id) holds its smallest site, and ranking roots by run id ranks the
 // clusters by label.  No workspace is used: the results go straight to the outputs.
 //
-// Latency bounds a call (barriers, and chains of dependent shared loads).  With links for
-// the first pairs, ranks from root bits and one scan for two segments a thread, one CTA
-// takes 26.6 us for 32^3 at p = 0.3 (36.9 with every pair united by its segment's thread
-// and ranks by blocks of run ids), a batch of 32 such lattices 29 us (89).
+// Latency bounds a call (barriers, chains of dependent shared loads, and the code fetched).
+// With links for the first pairs, ranks from root bits and one scan for two segments a
+// thread, one CTA takes 24.1 us for 32^3 at p = 0.3 (36.9 with every pair united by its
+// segment's thread and ranks by blocks of run ids), a batch of 32 such lattices 25 us (89).
 #include <cooperative_groups.h>
 
 #include <cstddef>
@@ -323,9 +323,9 @@ __global__ void __launch_bounds__(SNT, 1) k_small_label(const __grid_constant__ 
 // CTAs are separated by cluster barriers.
 //
 // Latency bounds a call here too.  A 32^3 lattice gives a CTA 64 segments, so the pairs
-// inside a CTA that links do not take are shared out by eighths of a segment: 20.6 us at
-// p = 0.3 and 22.5 at 0.45 (24.5 and 24.6 with all pairs counted, listed and united; 22.9
-// and 26.7 with one thread a segment).
+// inside a CTA that links do not take are shared out by nibbles of a segment: 20.5 us at
+// p = 0.3 and 0.45 (24.5 and 24.6 with all pairs counted, listed and united; 22.9 and 26.7
+// with one thread a segment).
 // ---------------------------------------------------------------------------------------
 // CTAs per lattice: 16 where the device co-schedules that many (a non-portable cluster
 // size), else 8 (the portable size); a template parameter of the kernel (CSB = log2).
