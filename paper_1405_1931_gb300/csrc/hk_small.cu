@@ -565,7 +565,7 @@ __global__ void __cluster_dims__(1 << CSB, 1, 1) __launch_bounds__(CNT, 1)
         }
     };
     static_assert(2 * CRUN_BITS + CS_BITS <= 32 && CS <= 32, "a listed pair packs into 32 bits");
-    {
+    if (total > 0) {                                 // CTA-uniform
         const int lcap = (local_cap > 0 && local_cap < total) ? local_cap : total;
         // the edges inside the CTA, one segment a thread: as in the tile pass a run's first
         // pair with a lower row is a store into its own node and a z pair whose site is
